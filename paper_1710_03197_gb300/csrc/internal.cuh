@@ -52,7 +52,8 @@ struct Chunk {
   int32_t bin;
   int32_t start;   // first sorted point
   int32_t count;   // points in this chunk
-  int32_t pad;
+  int32_t wmax;    // 3D: float bits of the largest sum of weight magnitudes of a cell (k_chunk_wmax)
+  int32_t slot;    // its partial tile: position in bin order (bin_chunk's index)
 };
 
 }  // namespace nufft

@@ -439,6 +439,18 @@ k_interp_chunk2d(const float2* __restrict__ grid_b, float2* __restrict__ y_b, co
 //     part above 2^20 of both components packed as two 16-bit fields of one
 //     word (|sum| <= 2^14 + 1024 each), and the remainders below 2^20 in one
 //     word each (|sum| <= 2048 * 2^19); rounding error at most 2^-35 B.
+//   3D chunks whose points are spread out use two words instead: the plan keeps
+//     W = the largest sum of weight magnitudes over the cells of the chunk's
+//     tile (k_chunk_wmax), so a cell's sum is also below B2 = W max|y|, and one
+//     int32 word per component holds 2^31 of range (S = 2^(31 - E2),
+//     B2 (1 + 2^-9) < 2^E2; the roundings of <= 2048 contributions fit in the
+//     margin).  A chunk does so only where its rounding step 2^(E2 - 31) is no
+//     larger than the three words' 2^(E - 34), so no result loses precision.
+//     A kooshball's outer tiles have B / B2 of 30 to 150 (a few points per
+//     cell, hundreds per tile); only its centre and its nearly empty tiles
+//     keep three words.  Two words cost two atomics and two conversions per
+//     tap where three cost three atomics and the split (about 20 instructions
+//     per tap): see k_gridding_chunk.
 // A chunk whose bound is not finite (an Inf or NaN sample) writes NaN.
 template <int D>
 struct Fix {
@@ -460,9 +472,24 @@ __device__ __forceinline__ float block_sum_fixed(float v, float* red) {
   return t;
 }
 
+// Largest v over the CTA (v >= 0; a NaN or Inf shows in the sum taken beside
+// it); every thread gets it.  red: 32 floats of shared scratch.
+__device__ __forceinline__ float block_max(float v, float* red) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  const int nw = blockDim.x >> 5;
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  float t = 0.f;
+  for (int w = 0; w < nw; ++w) t = fmaxf(t, red[w]);
+  __syncthreads();   // red free for reuse
+  return t;
+}
+
 struct ChunkScale {
   float S, inv;   // power-of-two scale and its inverse
   bool finite;
+  bool two;       // 3D: two words per cell
 };
 
 template <int D>
@@ -478,15 +505,35 @@ __device__ __forceinline__ ChunkScale chunk_scale(float ysum, const uint32_t* cm
   E = max(E, Fix<D>::kBits - 126);                   // keep S and 1/S normal floats
   cs.S = ldexpf(1.f, Fix<D>::kBits - E);
   cs.inv = ldexpf(1.f, E - Fix<D>::kBits);
+  cs.two = false;
   return cs;
 }
 
+// 3D: two words where W max|y| (wmax of the chunk, ymax of its samples) gives
+// a rounding step no larger than the three words' (see above).
+__device__ __forceinline__ void try_two_words(ChunkScale& cs, float wmax, float ymax, const uint32_t* cmax) {
+  const float B2 = wmax * ymax * (1.f + 0x1p-9f);
+  if (!cs.finite || !isfinite(B2)) return;
+  float cb = ymax * (1.f + 0x1p-9f);   // one contribution stays below 2^30 (round_int)
+#pragma unroll
+  for (int a = 0; a < 3; ++a) cb *= __uint_as_float(__ldg(&cmax[a]));
+  int E1 = 0, E2 = 0;
+  frexpf(cb, &E1);
+  frexpf(B2, &E2);
+  E2 = max(max(E2, E1 + 1), 31 - 126);
+  const float inv2 = ldexpf(1.f, E2 - 31);
+  if (inv2 > cs.inv) return;
+  cs.S = ldexpf(1.f, 31 - E2);
+  cs.inv = inv2;
+  cs.two = true;
+}
+
 // Add one contribution w (already scaled by S) to cell `cell`.
-//   D < 3: acc[0][cell] += rn(Re w), acc[1][cell] += rn(Im w)
-//   D = 3: packed high parts in acc[0], remainders in acc[1], acc[2]
-template <int D>
+//   two words: acc[0][cell] += rn(Re w), acc[1][cell] += rn(Im w)
+//   three: packed high parts in acc[0], remainders in acc[1], acc[2]
+template <int WORDS>
 __device__ __forceinline__ void fix_add(int* acc, int ncell, int cell, float2 w) {
-  if (D < 3) {
+  if (WORDS == 2) {
     atomicAdd(&acc[cell], __float2int_rn(w.x));
     atomicAdd(&acc[ncell + cell], __float2int_rn(w.y));
   } else {
@@ -509,7 +556,7 @@ __device__ __forceinline__ void fix_add(int* acc, int ncell, int cell, float2 w)
 template <int D>
 __device__ __forceinline__ float2 fix_value(const int* acc, int ncell, int c, const ChunkScale& cs) {
   if (!cs.finite) return make_float2(__int_as_float(0x7fffffff), __int_as_float(0x7fffffff));
-  if (D < 3) return make_float2((float)acc[c] * cs.inv, (float)acc[ncell + c] * cs.inv);
+  if (D < 3 || cs.two) return make_float2((float)acc[c] * cs.inv, (float)acc[ncell + c] * cs.inv);
   const int w = acc[c];
   const int hre = (int)(short)(w & 0xffff);   // low field, sign-extended
   const int him = (w - hre) / 65536;
@@ -527,30 +574,249 @@ struct GridChunkCfg {
   static constexpr int kMinBlocks = D == 3 ? 2 : 4;
 };
 
+// Scatter of one chunk's points into the fixed-point tile (WORDS words per
+// cell).  Consecutive points of the chunk share a warp instruction: the plan
+// orders each chunk so that every aligned group of per_warp points covers
+// disjoint shared-memory bank windows (see the bank-order kernel in plan.cu).
 // TF > 0: every tile edge is TF and every J is JF, so the padded-tile pitches
 // are compile-time constants and the neighbour loops unroll into fixed
 // shared-memory offsets.
+template <int D, int JF, int TF, int WORDS>
+__device__ __forceinline__ void scatter_chunk(int* acc, const int ncell, const float2* __restrict__ y, const Chunk& ch,
+                                              const Points& P, const Geom& g, const int (&org)[kMaxDim], const float S) {
+  constexpr int PF = TF > 0 ? TF + JF - 1 : 0;   // padded edge when fixed
+  const int G = JF > 0 ? JF : g.J[D - 1];
+  const int lane = threadIdx.x & 31;
+  const int per_warp = 32 / G;
+  const int sub = lane / G;
+  const int l = lane - sub * G;
+  const int warp = threadIdx.x >> 5;
+  const int nwarps = blockDim.x >> 5;
+  const int P1 = D > 1 ? (TF > 0 ? PF : g.P[1]) : 1;
+  const int P2 = D > 2 ? (TF > 0 ? PF : g.P[2]) : 1;
+  if (sub >= per_warp) return;
+  const int stepq = nwarps * per_warp;
+  int q = warp * per_warp + sub;
+  // 1D: the dependent load (sample through the permutation) runs one point
+  // ahead; 3D has enough work per point to hide it and no registers to spare.
+  float2 y_next = make_float2(0.f, 0.f);
+  if (D < 3 && q < ch.count) y_next = __ldg(&y[P.perm[(int64_t)ch.start + q]]);
+  for (; q < ch.count; q += stepq) {
+    const int64_t i = (int64_t)ch.start + q;
+    float2 yv;
+    if (D < 3) {
+      yv = y_next;
+      if (q + stepq < ch.count) y_next = __ldg(&y[P.perm[i + stepq]]);
+    } else {
+      yv = __ldg(&y[P.perm[i]]);
+    }
+    yv = cscale(yv, S);
+    const int ll = P.kf[(int64_t)(D - 1) * P.M + i] - org[D - 1] + l;
+    const float2 cl = P.coef[P.coef_off[D - 1] + (int64_t)l * P.M + i];
+    const float2 yl = cmulc(cl, yv);  // conj(c_last) * y
+    if (D == 1) {
+      fix_add<WORDS>(acc, ncell, ll, yl);
+    } else {
+      const int l0 = P.kf[i] - org[0];
+      const int l1 = P.kf[P.M + i] - org[1];
+      const int J0 = JF > 0 ? JF : g.J[0];
+      const int J1 = JF > 0 ? JF : g.J[1];
+      float2 c1v[JF > 0 ? JF : kMaxJ];
+#pragma unroll
+      for (int j1 = 0; j1 < (JF > 0 ? JF : kMaxJ); ++j1) {
+        if (JF == 0 && j1 >= J1) break;
+        c1v[j1] = P.coef[P.coef_off[1] + (int64_t)j1 * P.M + i];
+      }
+      constexpr int kU0 = TF > 0 ? JF : 1;
+#pragma unroll kU0
+      for (int j0 = 0; j0 < J0; ++j0) {
+        const float2 c0 = P.coef[P.coef_off[0] + (int64_t)j0 * P.M + i];
+        const float2 w0 = cmulc(c0, yl);
+        const int rowbase = ((l0 + j0) * P1 + l1) * P2 + ll;
+#pragma unroll
+        for (int j1 = 0; j1 < (JF > 0 ? JF : kMaxJ); ++j1) {
+          if (JF == 0 && j1 >= J1) break;
+          fix_add<WORDS>(acc, ncell, rowbase + j1 * P2, cmulc(c1v[j1], w0));
+        }
+      }
+    }
+  }
+}
+
+// 3D chunk pass with every J = JF (4 to 7): as k_gridding_chunk, but a chunk
+// that sums in two words keeps its samples in shared memory (they are gathered
+// once, for the scale; the third word's space holds them), and every warp keeps
+// the next round's coefficients in flight while it scatters this one's: lane l
+// of a point loads the l-th coefficient of each axis into registers a round
+// ahead, and the axis-0 and axis-1 ones are passed to the point's other lanes
+// through a per-warp strip of shared memory.  A chunk that needs three words
+// takes scatter_chunk.
+template <int JF>
+struct Chunk3dCfg {
+  static constexpr int kThreads = 512;
+  static constexpr int kPerWarp = 32 / JF;
+  static constexpr int kStrip = 2 * JF * kPerWarp;   // float2 per warp
+  static size_t smem(int64_t cells) {   // two words, samples and strips, or three words
+    return std::max((size_t)cells * 2 * sizeof(int) +
+                        ((size_t)kChunkPoints[3] + (kThreads / 32) * kStrip) * sizeof(float2),
+                    (size_t)cells * 3 * sizeof(int));
+  }
+};
+
+// rn(x) as an integer for |x| < 1.2e9 on the FP32 and integer pipes: three
+// additions and a shift-add, against one F2I, which the conversion unit issues
+// at one warp per two cycles and SM.  t holds x rounded to a multiple of 512
+// (its ulp), l the remainder plus 1.5 * 2^23, exactly rounded, and the mantissa
+// of kT is chosen so that the constant bits of 512 t + l cancel modulo 2^32:
+// 512 * 0x5a6000 + 0x4b400000 = 2^32.
+__device__ __forceinline__ int round_int(float x) {
+  const float kT = __int_as_float(0x4f800000 + 0x5a6000 );   // 2^32 (1 + 0x5a6000 / 2^23): ulp 512
+  const float t = __fadd_rn(x, kT);
+  const float u = __fsub_rn(t, __fadd_rn(kT, 12582912.0f));   // multiple of 512, less 1.5 * 2^23: exact
+  const float l = __fsub_rn(x, u);
+  return (__float_as_int(t) << 9) + __float_as_int(l);
+}
+
+template <int JF, int TF>
+__device__ __forceinline__ void scatter_chunk3d(int* acc, const int ncell, const float2* s_y, float2* strip,
+                                                const Chunk& ch, const Points& P, const Geom& g,
+                                                const int (&org)[kMaxDim], const float S) {
+  constexpr int PF = TF > 0 ? TF + JF - 1 : 0;
+  constexpr int PW = Chunk3dCfg<JF>::kPerWarp;
+  const int P1 = TF > 0 ? PF : g.P[1];
+  const int P2 = TF > 0 ? PF : g.P[2];
+  const int lane = threadIdx.x & 31;
+  const int sub = lane / JF;
+  const int l = lane - sub * JF;
+  const int step = (Chunk3dCfg<JF>::kThreads / 32) * PW;
+  const int64_t M = P.M;
+  const float2* pc0 = P.coef + P.coef_off[0] + (int64_t)l * M + ch.start;
+  const float2* pc1 = P.coef + P.coef_off[1] + (int64_t)l * M + ch.start;
+  const float2* pc2 = P.coef + P.coef_off[2] + (int64_t)l * M + ch.start;
+  const int32_t* pk = P.kf + ch.start;
+  int qb = (threadIdx.x >> 5) * PW;
+  bool act = sub < PW && qb + sub < ch.count;
+  float2 n0 = make_float2(0.f, 0.f), n1 = n0, n2 = n0;
+  int k0 = 0, k1 = 0, k2 = 0;
+  if (act) {
+    const int q = qb + sub;
+    n0 = pc0[q]; n1 = pc1[q]; n2 = pc2[q];
+    k0 = pk[q]; k1 = pk[M + q]; k2 = pk[2 * M + q];
+  }
+  for (; qb < ch.count; qb += step) {   // warp-uniform
+    const bool cur = act;
+    __syncwarp();   // the strip's readers of the previous round are done
+    float2 yl = make_float2(0.f, 0.f);
+    int base = 0;
+    if (cur) {
+      strip[l * PW + sub] = n0;
+      strip[(JF + l) * PW + sub] = n1;
+      yl = cmulc(n2, cscale(s_y[qb + sub], S));   // conj(c_last) * y
+      base = ((k0 - org[0]) * P1 + k1 - org[1]) * P2 + k2 - org[2] + l;
+    }
+    const int qn = qb + step + sub;
+    act = sub < PW && qn < ch.count;
+    if (act) {
+      n0 = pc0[qn]; n1 = pc1[qn]; n2 = pc2[qn];
+      k0 = pk[qn]; k1 = pk[M + qn]; k2 = pk[2 * M + qn];
+    }
+    __syncwarp();
+    if (cur) {
+      float2 c1v[JF];
+#pragma unroll
+      for (int j1 = 0; j1 < JF; ++j1) c1v[j1] = strip[(JF + j1) * PW + sub];
+#pragma unroll
+      for (int j0 = 0; j0 < JF; ++j0) {
+        const float2 w0 = cmulc(strip[j0 * PW + sub], yl);
+        int* row = acc + base + j0 * P1 * P2;
+#pragma unroll
+        for (int j1 = 0; j1 < JF; ++j1) {
+          const float2 w = cmulc(c1v[j1], w0);
+          int* cell = row + j1 * P2;
+          // the conversion unit takes the real parts and half of the imaginary
+          // ones, the FP32 pipe the rest
+          atomicAdd(cell, __float2int_rn(w.x));
+          atomicAdd(cell + ncell, (j1 & 1) ? round_int(w.y) : __float2int_rn(w.y));
+        }
+      }
+    }
+  }
+}
+
+template <int JF, int TF>
+__global__ void __launch_bounds__(Chunk3dCfg<JF>::kThreads, 2)
+k_gridding_chunk3d(const float2* __restrict__ y_b, float2* __restrict__ tiles_b, const Chunk* __restrict__ chunks,
+                   const Points P, const Geom g, int64_t ybs, int64_t tbs) {
+  constexpr int PF = TF > 0 ? TF + JF - 1 : 0;
+  extern __shared__ int acc[];
+  __shared__ float red[32];
+  const float2* __restrict__ y = y_b + (int64_t)blockIdx.y * ybs;
+  float2* __restrict__ out = tiles_b + (int64_t)blockIdx.y * tbs;
+  const int ncell = TF > 0 ? PF * PF * PF : (int)g.padded_cells;
+  float2* s_y = reinterpret_cast<float2*>(acc + 2 * ncell);   // 8-byte aligned: 2 * ncell words
+  float2* strip = s_y + kChunkPoints[3] + (threadIdx.x >> 5) * Chunk3dCfg<JF>::kStrip;
+  const Chunk ch = chunks[blockIdx.x];
+  out += (int64_t)ch.slot * g.padded_cells;
+  float part = 0.f, ymax = 0.f;
+  for (int q = threadIdx.x; q < ch.count; q += blockDim.x) {
+    const float2 v = __ldg(&y[P.perm[(int64_t)ch.start + q]]);
+    s_y[q] = v;
+    const float a = fabsf(v.x), b = fabsf(v.y);
+    part += a + b;
+    // |v| <= sqrt 2 max(a, b) and <= a + b; either bounds the contributions
+    ymax = fmaxf(ymax, fminf(a + b, 1.41421368f * fmaxf(a, b)));
+  }
+  for (int c = threadIdx.x; c < 2 * ncell; c += blockDim.x) acc[c] = 0;
+  // the sums also order the zeroing and s_y before their use
+  ChunkScale cs = chunk_scale<3>(block_sum_fixed(part, red), P.cmax);
+  try_two_words(cs, __int_as_float(ch.wmax), block_max(ymax, red), P.cmax);
+  int org[kMaxDim];
+  {
+    int rem = ch.bin;
+    for (int a = 2; a >= 0; --a) {
+      org[a] = (rem % g.nb[a]) * g.T[a];
+      rem /= g.nb[a];
+    }
+  }
+  if (cs.two) {   // CTA-uniform
+    scatter_chunk3d<JF, TF>(acc, ncell, s_y, strip, ch, P, g, org, cs.S);
+  } else if (cs.finite) {
+    for (int c = threadIdx.x; c < ncell; c += blockDim.x) acc[2 * ncell + c] = 0;   // over the samples
+    __syncthreads();
+    scatter_chunk<3, JF, TF, 3>(acc, ncell, y, ch, P, g, org, cs.S);
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < ncell; c += blockDim.x) out[c] = fix_value<3>(acc, ncell, c, cs);
+}
+
+// 1D chunk pass, and the 3D one for the J that k_gridding_chunk3d does not take
+// (2D: k_gridding_chunk_staged).
 template <int D, int JF, int TF>
 __global__ void __launch_bounds__(GridChunkCfg<D, JF>::kThreads, GridChunkCfg<D, JF>::kMinBlocks)
 k_gridding_chunk(const float2* __restrict__ y_b, float2* __restrict__ tiles_b, const Chunk* __restrict__ chunks,
                  const Points P, const Geom g, int64_t ybs, int64_t tbs) {
+  static_assert(D != 2, "2D has its own kernel");
   static_assert(TF == 0 || JF > 0, "a fixed tile needs a fixed J");
   constexpr int PF = TF > 0 ? TF + JF - 1 : 0;   // padded edge when fixed
   extern __shared__ int acc[];
   __shared__ float red[32];
   const float2* __restrict__ y = y_b + (int64_t)blockIdx.y * ybs;
   float2* __restrict__ tiles = tiles_b + (int64_t)blockIdx.y * tbs;
-  const int ncell = TF > 0 ? (D == 1 ? PF : (D == 2 ? PF * PF : PF * PF * PF)) : (int)g.padded_cells;
+  const int ncell = TF > 0 ? (D == 1 ? PF : PF * PF * PF) : (int)g.padded_cells;
   const Chunk ch = chunks[blockIdx.x];
   for (int c = threadIdx.x; c < Fix<D>::kWords * ncell; c += blockDim.x) acc[c] = 0;
 
-  // the chunk's scale (the sum also orders the zeroing above before the atomics)
-  float part = 0.f;
+  // the chunk's scale (the sums also order the zeroing above before the atomics)
+  float part = 0.f, ymax = 0.f;
   for (int q = threadIdx.x; q < ch.count; q += blockDim.x) {
     const float2 v = __ldg(&y[P.perm[(int64_t)ch.start + q]]);
-    part += fabsf(v.x) + fabsf(v.y);
+    const float a = fabsf(v.x), b = fabsf(v.y);
+    part += a + b;
+    // |v| <= sqrt 2 max(a, b) and <= a + b; either bounds the contributions
+    if (D == 3) ymax = fmaxf(ymax, fminf(a + b, 1.41421368f * fmaxf(a, b)));
   }
-  const ChunkScale cs = chunk_scale<D>(block_sum_fixed(part, red), P.cmax);
+  ChunkScale cs = chunk_scale<D>(block_sum_fixed(part, red), P.cmax);
+  if (D == 3) try_two_words(cs, __int_as_float(ch.wmax), block_max(ymax, red), P.cmax);
 
   // tile origin of this chunk's bin
   int org[kMaxDim];
@@ -561,79 +827,12 @@ k_gridding_chunk(const float2* __restrict__ y_b, float2* __restrict__ tiles_b, c
       rem /= g.nb[a];
     }
   }
-  const int G = JF > 0 ? JF : g.J[D - 1];
-  const int lane = threadIdx.x & 31;
-  const int per_warp = 32 / G;
-  const int sub = lane / G;
-  const int l = lane - sub * G;
-  const int warp = threadIdx.x >> 5;
-  const int nwarps = blockDim.x >> 5;
-  const int P1 = D > 1 ? (TF > 0 ? PF : g.P[1]) : 1;
-  const int P2 = D > 2 ? (TF > 0 ? PF : g.P[2]) : 1;
-
-  // Consecutive points of the chunk share a warp instruction: the plan orders
-  // each chunk so that every aligned group of per_warp points covers disjoint
-  // shared-memory bank windows (see the bank-order kernel in plan.cu).
-  if (sub < per_warp && cs.finite) {
-    const int stepq = nwarps * per_warp;
-    int q = warp * per_warp + sub;
-    // 1D/2D: the dependent load (sample through the permutation) runs one
-    // point ahead; 3D has enough work per point to hide it and no registers
-    // to spare.
-    float2 y_next = make_float2(0.f, 0.f);
-    if (D < 3 && q < ch.count) y_next = __ldg(&y[P.perm[(int64_t)ch.start + q]]);
-    for (; q < ch.count; q += stepq) {
-      const int64_t i = (int64_t)ch.start + q;
-      float2 yv;
-      if (D < 3) {
-        yv = y_next;
-        if (q + stepq < ch.count) y_next = __ldg(&y[P.perm[i + stepq]]);
-      } else {
-        yv = __ldg(&y[P.perm[i]]);
-      }
-      yv = cscale(yv, cs.S);
-      const int ll = P.kf[(int64_t)(D - 1) * P.M + i] - org[D - 1] + l;
-      const float2 cl = P.coef[P.coef_off[D - 1] + (int64_t)l * P.M + i];
-      const float2 yl = cmulc(cl, yv);  // conj(c_last) * y
-      if (D == 1) {
-        fix_add<D>(acc, ncell, ll, yl);
-      } else if (D == 2) {
-        const int l0 = P.kf[i] - org[0];
-        const int J0 = JF > 0 ? JF : g.J[0];
-#pragma unroll
-        for (int j0 = 0; j0 < (JF > 0 ? JF : kMaxJ); ++j0) {
-          if (JF == 0 && j0 >= J0) break;
-          const float2 c0 = P.coef[P.coef_off[0] + (int64_t)j0 * P.M + i];
-          fix_add<D>(acc, ncell, (l0 + j0) * P1 + ll, cmulc(c0, yl));
-        }
-      } else {
-        const int l0 = P.kf[i] - org[0];
-        const int l1 = P.kf[P.M + i] - org[1];
-        const int J0 = JF > 0 ? JF : g.J[0];
-        const int J1 = JF > 0 ? JF : g.J[1];
-        float2 c1v[JF > 0 ? JF : kMaxJ];
-#pragma unroll
-        for (int j1 = 0; j1 < (JF > 0 ? JF : kMaxJ); ++j1) {
-          if (JF == 0 && j1 >= J1) break;
-          c1v[j1] = P.coef[P.coef_off[1] + (int64_t)j1 * P.M + i];
-        }
-        constexpr int kU0 = TF > 0 ? JF : 1;
-#pragma unroll kU0
-        for (int j0 = 0; j0 < J0; ++j0) {
-          const float2 c0 = P.coef[P.coef_off[0] + (int64_t)j0 * P.M + i];
-          const float2 w0 = cmulc(c0, yl);
-          const int rowbase = ((l0 + j0) * P1 + l1) * P2 + ll;
-#pragma unroll
-          for (int j1 = 0; j1 < (JF > 0 ? JF : kMaxJ); ++j1) {
-            if (JF == 0 && j1 >= J1) break;
-            fix_add<D>(acc, ncell, rowbase + j1 * P2, cmulc(c1v[j1], w0));
-          }
-        }
-      }
-    }
+  if (cs.finite) {   // CTA-uniform
+    if (D < 3 || cs.two) scatter_chunk<D, JF, TF, 2>(acc, ncell, y, ch, P, g, org, cs.S);
+    else scatter_chunk<D, JF, TF, 3>(acc, ncell, y, ch, P, g, org, cs.S);
   }
   __syncthreads();
-  float2* out = tiles + (int64_t)blockIdx.x * g.padded_cells;
+  float2* out = tiles + (int64_t)ch.slot * g.padded_cells;
   for (int c = threadIdx.x; c < ncell; c += blockDim.x) out[c] = fix_value<D>(acc, ncell, c, cs);
 }
 
@@ -1011,7 +1210,7 @@ k_gridding_chunk_staged(const float2* __restrict__ y_b, float2* __restrict__ til
     }
   }
   __syncthreads();
-  float2* out = tiles + (int64_t)blockIdx.x * g.padded_cells;
+  float2* out = tiles + (int64_t)ch.slot * g.padded_cells;
   for (int c = threadIdx.x; c < ncell; c += blockDim.x) out[c] = fix_value<2>(acc, ncell, c, cs);
 }
 
@@ -1111,6 +1310,24 @@ cudaError_t interp_d(const nufft_plan_t* p, const float2* grid, float2* y, int n
   return cudaGetLastError();
 }
 
+cudaError_t launch_chunks3d(const nufft_plan_t* p, const float2* y, float2* tiles, dim3 gd, int J, int64_t ybs,
+                            int64_t tbs) {
+  const bool t16 = p->g.T[0] == 16 && p->g.T[1] == 16 && p->g.T[2] == 16;
+  auto go = [&](auto kern, size_t smem) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<gd, 512, smem, p->stream>>>(y, tiles, p->chunks, points_view(p), p->g, ybs, tbs);
+    return cudaGetLastError();
+  };
+  const int64_t cells = p->g.padded_cells;
+  switch (J) {
+    case 4: return go(t16 ? k_gridding_chunk3d<4, 16> : k_gridding_chunk3d<4, 0>, Chunk3dCfg<4>::smem(cells));
+    case 5: return go(t16 ? k_gridding_chunk3d<5, 16> : k_gridding_chunk3d<5, 0>, Chunk3dCfg<5>::smem(cells));
+    case 6: return go(t16 ? k_gridding_chunk3d<6, 16> : k_gridding_chunk3d<6, 0>, Chunk3dCfg<6>::smem(cells));
+    default: return go(t16 ? k_gridding_chunk3d<7, 16> : k_gridding_chunk3d<7, 0>, Chunk3dCfg<7>::smem(cells));
+  }
+}
+
 // Chunk pass of V^H: one CTA per (chunk, batch element), partial tiles out.
 // FUSED (2D only): y is the oversampled spectrum and the pass computes V^H V.
 template <int D, bool FUSED = false>
@@ -1133,10 +1350,11 @@ cudaError_t launch_chunks(const nufft_plan_t* p, const float2* y, float2* tiles,
     static_assert(!FUSED, "the fused V^H V pass is 2D only");
     const size_t smem = (size_t)p->g.padded_cells * Fix<D>::kWords * sizeof(int);
     constexpr int NT = GridChunkCfg<D, 6>::kThreads;
-    bool t16 = D == 3;
-    for (int a = 0; a < D; ++a) t16 = t16 && p->g.T[a] == 16;
-    auto kern = j6 ? (t16 ? k_gridding_chunk<D, 6, (D == 3 ? 16 : 0)> : k_gridding_chunk<D, 6, 0>)
-                   : k_gridding_chunk<D, 0, 0>;
+    if constexpr (D == 3) {
+      const int J = all_j_equal(p->g, p->g.J[0]) ? p->g.J[0] : 0;
+      if (J >= 4 && J <= 7) return launch_chunks3d(p, y, tiles, gd, J, ybs, tbs);
+    }
+    auto kern = D == 1 && j6 ? k_gridding_chunk<D, (D == 1 ? 6 : 0), 0> : k_gridding_chunk<D, 0, 0>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<gd, NT, smem, p->stream>>>(y, tiles, p->chunks, P, p->g, ybs, tbs);

@@ -454,6 +454,62 @@ __global__ void k_coef_max(const float2* coef, int64_t M, int d, int J0, int J1,
   }
 }
 
+// 3D: W of every chunk, an upper bound on the sum over the chunk's points of
+// the weight magnitude |c_0| |c_1| |c_2| at any one cell of its padded tile,
+// for the gridding's two-word mode (interp.cu).  The weights are rounded up to
+// multiples of 2^-20 cbound and summed as unsigned integers (at most 2048
+// points of at most 2^20 + 1: no overflow), so W does not depend on the order
+// of the atomics.  Lane layout and bank order are the gridding's; one atomic
+// and no samples, so about a third of its time.
+__global__ void __launch_bounds__(512)
+k_chunk_wmax(Chunk* chunks, const int32_t* kf, const float2* coef, int64_t off1, int64_t off2, int64_t M, const Geom g,
+             const uint32_t* cmax) {
+  extern __shared__ uint32_t wacc[];
+  __shared__ uint32_t top;
+  static_assert(kChunkPoints[3] <= 2048, "32-bit sums");
+  const Chunk ch = chunks[blockIdx.x];
+  const int ncell = (int)g.padded_cells;
+  for (int c = threadIdx.x; c < ncell; c += blockDim.x) wacc[c] = 0;
+  if (threadIdx.x == 0) top = 0;
+  __syncthreads();
+  const float cb = __uint_as_float(cmax[0]) * __uint_as_float(cmax[1]) * __uint_as_float(cmax[2]) * (1.f + 0x1p-20f);
+  const float sc = cb > 0.f ? 0x1p20f / cb : 0.f;
+  int org[kMaxDim];
+  {
+    int rem = ch.bin;
+    for (int a = 2; a >= 0; --a) {
+      org[a] = (rem % g.nb[a]) * g.T[a];
+      rem /= g.nb[a];
+    }
+  }
+  const int G = g.J[2], lane = threadIdx.x & 31, per_warp = 32 / G, sub = lane / G, l = lane - sub * G;
+  if (sub < per_warp) {
+    for (int q = (threadIdx.x >> 5) * per_warp + sub; q < ch.count; q += (blockDim.x >> 5) * per_warp) {
+      const int64_t i = (int64_t)ch.start + q;
+      const float2 c2 = coef[off2 + (int64_t)l * M + i];
+      const float w2 = sqrtf(c2.x * c2.x + c2.y * c2.y) * sc;
+      const int l0 = kf[i] - org[0], l1 = kf[M + i] - org[1], ll = kf[2 * M + i] - org[2] + l;
+      for (int j0 = 0; j0 < g.J[0]; ++j0) {
+        const float2 c0 = coef[(int64_t)j0 * M + i];
+        const float w0 = sqrtf(c0.x * c0.x + c0.y * c0.y) * w2;
+        for (int j1 = 0; j1 < g.J[1]; ++j1) {
+          const float2 c1 = coef[off1 + (int64_t)j1 * M + i];
+          const float w = sqrtf(c1.x * c1.x + c1.y * c1.y) * w0;
+          atomicAdd(&wacc[((l0 + j0) * g.P[1] + l1 + j1) * g.P[2] + ll],
+                    min((uint32_t)ceilf(w * (1.f + 0x1p-20f)), (1u << 20) + 1u));
+        }
+      }
+    }
+  }
+  __syncthreads();
+  uint32_t m = 0;
+  for (int c = threadIdx.x; c < ncell; c += blockDim.x) m = max(m, wacc[c]);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) atomicMax(&top, m);
+  __syncthreads();
+  if (threadIdx.x == 0) chunks[blockIdx.x].wmax = __float_as_int(__uint2float_ru(top) * (0x1p-20f * cb) * (1.f + 0x1p-20f));
+}
+
 // Order each chunk's points for the gridding kernel.  Lane groups of J_last
 // lanes handle one point each and G = 32 / J_last consecutive points share a
 // warp instruction; point p's atomics for neighbour tap (j_0..j_{d-1}) land on
@@ -656,12 +712,24 @@ int build_points(nufft_plan_t* p, const float* om) {
       c.bin = (int32_t)b;
       c.start = s0;
       c.count = std::min<int32_t>(kChunkPoints[d], bs[b + 1] - s0);
-      c.pad = 0;
+      c.wmax = 0;
+      c.slot = (int32_t)ch.size();
       ch.push_back(c);
     }
   }
   bc[g.nbins] = (int32_t)ch.size();
   const int64_t nch = (int64_t)ch.size();
+  // The chunk list in launch order: the longest chunks first (stable), so that
+  // the last wave of a 3D pass holds short ones.  A kooshball's dense chunks sit
+  // in the middle of the bin order; partial tiles keep that order (slot).
+  if (d == 3) {
+    std::vector<int32_t> pos(kChunkPoints[3] + 2, 0);
+    for (const Chunk& c : ch) ++pos[kChunkPoints[3] - c.count + 1];
+    for (size_t i = 1; i < pos.size(); ++i) pos[i] += pos[i - 1];
+    std::vector<Chunk> sorted(ch.size());
+    for (const Chunk& c : ch) sorted[pos[kChunkPoints[3] - c.count]++] = c;
+    ch.swap(sorted);
+  }
   if (nch > p->chunk_cap) {   // grow the chunk list and the partial tiles (and the batched ones, lazily)
     drop_graphs(p);
     for (void* b : {(void*)p->chunks, (void*)p->tiles, (void*)p->btiles})
@@ -752,6 +820,13 @@ int build_points(nufft_plan_t* p, const float* om) {
     k_coef_max<<<(unsigned)std::min<int64_t>(1024, (M * d + 255) / 256), 256, 0, st>>>(
         p->coef, M, d, g.J[0], d > 1 ? g.J[1] : 0, d > 2 ? g.J[2] : 0, p->cmax);
     NUFFT_CUDA_TRY(p, cudaGetLastError());
+    if (d == 3 && nch > 0) {
+      const size_t smem = (size_t)g.padded_cells * sizeof(uint32_t);
+      NUFFT_CUDA_TRY(p, cudaFuncSetAttribute(k_chunk_wmax, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      k_chunk_wmax<<<(unsigned)nch, 512, smem, st>>>(p->chunks, p->kf, p->coef, p->coef_off[1], p->coef_off[2], M, g,
+                                                     p->cmax);
+      NUFFT_CUDA_TRY(p, cudaGetLastError());
+    }
     if (p->dcoef) {
       k_coefficients<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(
           p->om_sorted, 1, g, M, p->perm, p->s64, D, p->Tinv, nullptr, p->dcoef, p->coef_off[0], p->coef_off[1],
