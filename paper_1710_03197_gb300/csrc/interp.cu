@@ -244,100 +244,189 @@ k_interp_chunk(const float2* __restrict__ grid_b, float2* __restrict__ y_b, cons
   }
 }
 
-// 3D, J = 6, 16^3 tiles: as k_interp_chunk, and the point data are staged too,
-// kSub points at a time (two threads per point: first neighbours, the 18
-// coefficients, the permutation), so every global load of point data is a
-// coalesced row of consecutive points and the gathers read only shared
-// memory.  kSub = 160 points fill two rounds of the 16 warps' lane groups and
-// keep two CTAs per SM (74 KB tile + 25 KB point data each).
-constexpr int kSub3 = 160;
-__global__ void __launch_bounds__(512, 2)
+// Packed pairs of floats: two FP32 multiply-adds in one instruction (fma.rn.f32x2),
+// each rounded as fmaf.  The FP32 pipe takes it at half rate, so it saves issue
+// slots, not pipe time: the gathers below issue two loads and two of these per
+// complex tap where four fmaf were.
+struct f32x2 {
+  unsigned long long v;
+};
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+
+// 3D with every J = JF (4 to 7): as k_interp_chunk, and every warp keeps the next
+// round's point data in flight while it gathers this one's, with no barrier
+// between rounds: lane l of a point loads the l-th coefficient of each axis into
+// registers a round ahead; the axis-0 and axis-1 ones reach the point's other
+// lanes through a per-warp strip of shared memory.  The J axis-1 taps of a row
+// are taken two at a time (fma2 on the pairs (re_j, re_j+1) and (im_j, im_j+1)).
+template <int JF>
+struct Chunk3dCfg {
+  static constexpr int kThreads = 512;
+  static constexpr int kPerWarp = 32 / JF;
+  static constexpr int kStrip = 2 * JF * kPerWarp;   // float2 per warp
+  // gridding: two words per cell, the samples and the strips, or three words
+  static size_t smem_gridding(int64_t cells) {
+    return std::max((size_t)cells * 2 * sizeof(int) +
+                        ((size_t)kChunkPoints[3] + (kThreads / 32) * kStrip) * sizeof(float2),
+                    (size_t)cells * 3 * sizeof(int));
+  }
+  static size_t smem_interp(int64_t cells) {
+    return (size_t)cells * 2 * sizeof(float) + (size_t)(kThreads / 32) * kStrip * sizeof(float2);
+  }
+};
+
+template <int JF, int TF>
+__global__ void __launch_bounds__(Chunk3dCfg<JF>::kThreads, 2)
 k_interp_chunk3d(const float2* __restrict__ grid_b, float2* __restrict__ y_b, const Chunk* __restrict__ chunks,
                  const Points P, const Geom g, int64_t gbs, int64_t ybs) {
-  constexpr int JF = 6, PF = 21, ncell = PF * PF * PF;
+  constexpr int PF = TF > 0 ? TF + JF - 1 : 0;
+  constexpr int PW = Chunk3dCfg<JF>::kPerWarp;
   extern __shared__ float tile[];
   const float2* __restrict__ grid = grid_b + (int64_t)blockIdx.y * gbs;
   float2* __restrict__ y = y_b + (int64_t)blockIdx.y * ybs;
+  const int P0 = TF > 0 ? PF : g.P[0];
+  const int P1 = TF > 0 ? PF : g.P[1];
+  const int P2 = TF > 0 ? PF : g.P[2];
+  const int ncell = P0 * P1 * P2;
   float* gre = tile;
   float* gim = tile + ncell;
-  float2* s_c0 = reinterpret_cast<float2*>(tile + 2 * ncell);   // [JF][kSub3] (2 * ncell floats: 8-byte aligned)
-  float2* s_c1 = s_c0 + JF * kSub3;                              // [JF][kSub3]
-  float2* s_c2 = s_c1 + JF * kSub3;                              // [kSub3][JF]
-  int* s_k = reinterpret_cast<int*>(s_c2 + JF * kSub3);          // [3][kSub3]
-  int* s_p = s_k + 3 * kSub3;                                    // [kSub3]
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  // strip: c0 as float2 [JF][PW], then the real and the imaginary parts of c1,
+  // [PW][JF] floats each, so that a point's pairs are adjacent
+  float2* s_c0 = reinterpret_cast<float2*>(tile + 2 * ncell) + warp * Chunk3dCfg<JF>::kStrip;
+  float* s_x1 = reinterpret_cast<float*>(s_c0 + JF * PW);
+  float* s_y1 = s_x1 + JF * PW;
   const Chunk ch = chunks[blockIdx.x];
   int org[3];
   {
     int rem = ch.bin;
     for (int a = 2; a >= 0; --a) {
-      org[a] = (rem % g.nb[a]) * 16;
+      org[a] = (rem % g.nb[a]) * g.T[a];
       rem /= g.nb[a];
     }
   }
-  for (int c = threadIdx.x; c < ncell; c += blockDim.x) {
-    const int r2 = c % PF, r1 = (c / PF) % PF, r0 = c / (PF * PF);
-    const int64_t gi = (int64_t)wrapk(org[0] + r0, g.K[0]) * g.Kstride[0] +
-                       (int64_t)wrapk(org[1] + r1, g.K[1]) * g.Kstride[1] + wrapk(org[2] + r2, g.K[2]);
-    const float2 v = __ldg(&grid[gi]);
-    gre[c] = v.x;
-    gim[c] = v.y;
-  }
-  const int lane = threadIdx.x & 31;
-  const int per_warp = 32 / JF;
   const int sub = lane / JF;
   const int l = lane - sub * JF;
-  const int warp = threadIdx.x >> 5;
-  const int nwarps = blockDim.x >> 5;
-  for (int s0 = 0; s0 < ch.count; s0 += kSub3) {
-    const int cnt = min(kSub3, ch.count - s0);
-    __syncthreads();   // the tile is staged; the previous sub-chunk's data are consumed
-    {
-      // two threads per point: half 0 loads c0 and the first neighbours, half 1 c1, c2 and the permutation
-      const int q = threadIdx.x % kSub3, half = threadIdx.x / kSub3;
-      if (half < 2 && q < cnt) {
-        const int64_t i = (int64_t)ch.start + s0 + q;
-        if (half == 0) {
+  constexpr int step = (Chunk3dCfg<JF>::kThreads / 32) * PW;
+  const int64_t M = P.M;
+  const float2* pc0 = P.coef + P.coef_off[0] + (int64_t)l * M + ch.start;
+  const float2* pc1 = P.coef + P.coef_off[1] + (int64_t)l * M + ch.start;
+  const float2* pc2 = P.coef + P.coef_off[2] + (int64_t)l * M + ch.start;
+  const int32_t* pk = P.kf + ch.start;
+  const int32_t* pp = P.perm + ch.start;
+  int qb = warp * PW;
+  bool act = sub < PW && qb + sub < ch.count;
+  float2 n0 = make_float2(0.f, 0.f), n1 = n0, n2 = n0;
+  int k0 = 0, k1 = 0, k2 = 0, m = 0;
+  if (act) {   // in flight while the tile is copied
+    const int q = qb + sub;
+    n0 = pc0[q]; n1 = pc1[q]; n2 = pc2[q];
+    k0 = pk[q]; k1 = pk[M + q]; k2 = pk[2 * M + q];
+    m = pp[q];
+  }
+  // the padded tile, kBatch cells of a thread in flight at a time (32-bit grid
+  // offsets: K^d <= 2^30)
+  constexpr int kBatch = 10;
+  for (int c0 = threadIdx.x; c0 < ncell; c0 += kBatch * Chunk3dCfg<JF>::kThreads) {
+    float2 v[kBatch];
 #pragma unroll
-          for (int r = 0; r < JF; ++r) s_c0[r * kSub3 + q] = P.coef[P.coef_off[0] + (int64_t)r * P.M + i];
-#pragma unroll
-          for (int a = 0; a < 3; ++a) s_k[a * kSub3 + q] = P.kf[(int64_t)a * P.M + i] - org[a];
-        } else {
-#pragma unroll
-          for (int r = 0; r < JF; ++r) s_c1[r * kSub3 + q] = P.coef[P.coef_off[1] + (int64_t)r * P.M + i];
-#pragma unroll
-          for (int r = 0; r < JF; ++r) s_c2[q * JF + r] = P.coef[P.coef_off[2] + (int64_t)r * P.M + i];
-          s_p[q] = P.perm[i];
-        }
+    for (int k = 0; k < kBatch; ++k) {
+      const int c = c0 + k * Chunk3dCfg<JF>::kThreads;
+      if (c < ncell) {
+        const int r2 = c % P2, r01 = c / P2, r1 = r01 % P1, r0 = r01 / P1;
+        const int gi = wrapk(org[0] + r0, g.K[0]) * (int)g.Kstride[0] + wrapk(org[1] + r1, g.K[1]) * (int)g.Kstride[1] +
+                       wrapk(org[2] + r2, g.K[2]);
+        v[k] = __ldg(&grid[gi]);
       }
     }
-    __syncthreads();
-    for (int qb = warp * per_warp; qb < cnt; qb += nwarps * per_warp) {
-      const int q = qb + sub;
-      const bool act = (sub < per_warp) && (q < cnt);
-      float2 part = make_float2(0.f, 0.f);
-      if (act) {
-        const int ll = s_k[2 * kSub3 + q] + l;
-        const int l0 = s_k[q], l1 = s_k[kSub3 + q];
-        float2 c1v[JF];
 #pragma unroll
-        for (int j1 = 0; j1 < JF; ++j1) c1v[j1] = s_c1[j1 * kSub3 + q];
-        float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int j0 = 0; j0 < JF; ++j0) {
-          const int rowbase = ((l0 + j0) * PF + l1) * PF + ll;
-          float2 acc1 = make_float2(0.f, 0.f);
-#pragma unroll
-          for (int j1 = 0; j1 < JF; ++j1) {
-            const int cell = rowbase + j1 * PF;
-            acc1 = cfma(c1v[j1], make_float2(gre[cell], gim[cell]), acc1);
-          }
-          acc = cfma(s_c0[j0 * kSub3 + q], acc1, acc);
-        }
-        part = cmul(s_c2[q * JF + l], acc);
+    for (int k = 0; k < kBatch; ++k) {
+      const int c = c0 + k * Chunk3dCfg<JF>::kThreads;
+      if (c < ncell) {
+        gre[c] = v[k].x;
+        gim[c] = v[k].y;
       }
-      const float2 tot = lane_group_sum<6>(part, sub * JF, JF);
-      if (act && l == 0) y[s_p[q]] = tot;
     }
+  }
+  __syncthreads();
+  for (; qb < ch.count; qb += step) {   // warp-uniform
+    const bool cur = act;
+    const float2 cl = n2;
+    const int mc = m;
+    int base = 0;
+    __syncwarp();   // the strip's readers of the previous round are done
+    if (cur) {
+      s_c0[l * PW + sub] = n0;
+      s_x1[sub * JF + l] = n1.x;
+      s_y1[sub * JF + l] = n1.y;
+      base = ((k0 - org[0]) * P1 + k1 - org[1]) * P2 + k2 - org[2] + l;
+    }
+    const int qn = qb + step + sub;
+    act = sub < PW && qn < ch.count;
+    if (act) {
+      n0 = pc0[qn]; n1 = pc1[qn]; n2 = pc2[qn];
+      k0 = pk[qn]; k1 = pk[M + qn]; k2 = pk[2 * M + qn];
+      m = pp[qn];
+    }
+    __syncwarp();
+    float2 part = make_float2(0.f, 0.f);
+    if (cur) {
+      float x1[JF], y1[JF];
+      if (JF & 1) {
+#pragma unroll
+        for (int j = 0; j < JF; ++j) {
+          x1[j] = s_x1[sub * JF + j];
+          y1[j] = s_y1[sub * JF + j];
+        }
+      } else {   // the pairs are 8-byte aligned
+#pragma unroll
+        for (int j = 0; j + 1 < JF; j += 2) {
+          const float2 vx = *reinterpret_cast<const float2*>(&s_x1[sub * JF + j]);
+          const float2 vy = *reinterpret_cast<const float2*>(&s_y1[sub * JF + j]);
+          x1[j] = vx.x; x1[j + 1] = vx.y;
+          y1[j] = vy.x; y1[j + 1] = vy.y;
+        }
+      }
+      float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int j0 = 0; j0 < JF; ++j0) {
+        const float* re = gre + base + j0 * P1 * P2;
+        const float* im = gim + base + j0 * P1 * P2;
+        f32x2 ar = pack2(0.f, 0.f), ai = ar;
+#pragma unroll
+        for (int j = 0; j + 1 < JF; j += 2) {
+          const f32x2 vx = pack2(re[j * P2], re[(j + 1) * P2]), vy = pack2(im[j * P2], im[(j + 1) * P2]);
+          const f32x2 cx = pack2(x1[j], x1[j + 1]), cy = pack2(y1[j], y1[j + 1]);
+          const f32x2 ny = pack2(-y1[j], -y1[j + 1]);
+          ar = fma2(cx, vx, ar);
+          ai = fma2(cx, vy, ai);
+          ar = fma2(ny, vy, ar);
+          ai = fma2(cy, vx, ai);
+        }
+        const float2 r2 = unpack2(ar), i2 = unpack2(ai);
+        float2 t = make_float2(r2.x + r2.y, i2.x + i2.y);
+        if (JF & 1) t = cfma(make_float2(x1[JF - 1], y1[JF - 1]), make_float2(re[(JF - 1) * P2], im[(JF - 1) * P2]), t);
+        acc = cfma(s_c0[j0 * PW + sub], t, acc);
+      }
+      part = cmul(cl, acc);
+    }
+    const float2 tot = lane_group_sum<JF>(part, sub * JF, JF);
+    if (cur && l == 0) y[mc] = tot;
   }
 }
 
@@ -651,18 +740,6 @@ __device__ __forceinline__ void scatter_chunk(int* acc, const int ncell, const f
 // ahead, and the axis-0 and axis-1 ones are passed to the point's other lanes
 // through a per-warp strip of shared memory.  A chunk that needs three words
 // takes scatter_chunk.
-template <int JF>
-struct Chunk3dCfg {
-  static constexpr int kThreads = 512;
-  static constexpr int kPerWarp = 32 / JF;
-  static constexpr int kStrip = 2 * JF * kPerWarp;   // float2 per warp
-  static size_t smem(int64_t cells) {   // two words, samples and strips, or three words
-    return std::max((size_t)cells * 2 * sizeof(int) +
-                        ((size_t)kChunkPoints[3] + (kThreads / 32) * kStrip) * sizeof(float2),
-                    (size_t)cells * 3 * sizeof(int));
-  }
-};
-
 // rn(x) as an integer for |x| < 1.2e9 on the FP32 and integer pipes: three
 // additions and a shift-add, against one F2I, which the conversion unit issues
 // at one warp per two cycles and SM.  t holds x rounded to a multiple of 512
@@ -1273,16 +1350,24 @@ cudaError_t interp_chunks(const nufft_plan_t* p, const float2* grid, float2* y, 
     kern<<<gd, kChunkPoints[2], smem, p->stream>>>(grid, y, p->chunks, P, p->g, p->Kprod, p->M);
     return cudaGetLastError();
   } else {
-    if (j6 && t16) {
-      const size_t smem = (size_t)21 * 21 * 21 * 2 * sizeof(float) +
-                          (size_t)kSub3 * (3 * 6 * sizeof(float2) + 4 * sizeof(int));
-      cudaError_t e = cudaFuncSetAttribute(k_interp_chunk3d, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      k_interp_chunk3d<<<gd, 512, smem, p->stream>>>(grid, y, p->chunks, P, p->g, p->Kprod, p->M);
-      return cudaGetLastError();
+    const int J = all_j_equal(p->g, p->g.J[0]) ? p->g.J[0] : 0;
+    if (J >= 4 && J <= 7) {
+      const int64_t cells = p->g.padded_cells;
+      auto go = [&](auto kern, size_t smem) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        kern<<<gd, 512, smem, p->stream>>>(grid, y, p->chunks, P, p->g, p->Kprod, p->M);
+        return cudaGetLastError();
+      };
+      switch (J) {
+        case 4: return go(t16 ? k_interp_chunk3d<4, 16> : k_interp_chunk3d<4, 0>, Chunk3dCfg<4>::smem_interp(cells));
+        case 5: return go(t16 ? k_interp_chunk3d<5, 16> : k_interp_chunk3d<5, 0>, Chunk3dCfg<5>::smem_interp(cells));
+        case 6: return go(t16 ? k_interp_chunk3d<6, 16> : k_interp_chunk3d<6, 0>, Chunk3dCfg<6>::smem_interp(cells));
+        default: return go(t16 ? k_interp_chunk3d<7, 16> : k_interp_chunk3d<7, 0>, Chunk3dCfg<7>::smem_interp(cells));
+      }
     }
     const size_t smem = (size_t)p->g.padded_cells * 2 * sizeof(float);
-    auto kern = j6 ? (t16 ? k_interp_chunk<D, 6, 16> : k_interp_chunk<D, 6, 0>) : k_interp_chunk<D, 0, 0>;
+    auto kern = k_interp_chunk<D, 0, 0>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<gd, InterpChunkCfg<D>::kThreads, smem, p->stream>>>(grid, y, p->chunks, P, p->g, p->Kprod, p->M);
@@ -1321,10 +1406,10 @@ cudaError_t launch_chunks3d(const nufft_plan_t* p, const float2* y, float2* tile
   };
   const int64_t cells = p->g.padded_cells;
   switch (J) {
-    case 4: return go(t16 ? k_gridding_chunk3d<4, 16> : k_gridding_chunk3d<4, 0>, Chunk3dCfg<4>::smem(cells));
-    case 5: return go(t16 ? k_gridding_chunk3d<5, 16> : k_gridding_chunk3d<5, 0>, Chunk3dCfg<5>::smem(cells));
-    case 6: return go(t16 ? k_gridding_chunk3d<6, 16> : k_gridding_chunk3d<6, 0>, Chunk3dCfg<6>::smem(cells));
-    default: return go(t16 ? k_gridding_chunk3d<7, 16> : k_gridding_chunk3d<7, 0>, Chunk3dCfg<7>::smem(cells));
+    case 4: return go(t16 ? k_gridding_chunk3d<4, 16> : k_gridding_chunk3d<4, 0>, Chunk3dCfg<4>::smem_gridding(cells));
+    case 5: return go(t16 ? k_gridding_chunk3d<5, 16> : k_gridding_chunk3d<5, 0>, Chunk3dCfg<5>::smem_gridding(cells));
+    case 6: return go(t16 ? k_gridding_chunk3d<6, 16> : k_gridding_chunk3d<6, 0>, Chunk3dCfg<6>::smem_gridding(cells));
+    default: return go(t16 ? k_gridding_chunk3d<7, 16> : k_gridding_chunk3d<7, 0>, Chunk3dCfg<7>::smem_gridding(cells));
   }
 }
 

@@ -1,0 +1,94 @@
+"""The passes that a size rule chooses, each side of it, against the FP64 oracle.
+
+FFT passes (line lengths, columns per CTA, eight or sixteen values per thread), the 3D
+chunk interpolation and tile reduction for every J they are built for, on tiles that are
+not 16 wide and with point counts at the edges of a round, and the batched 2D kernels.
+
+Tolerances: an FFT line of 256 points has 8 radix-2 levels, each with at most about
+1.5 * 2^-24 of relative rounding in the 2-norm; three axes give 3 * 8 * 1.5 * 2^-24 =
+2.1e-6 if all errors added up: 2e-6.  Interpolation and gridding: about eight roundings of
+2^-24 per contribution: 1e-6.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL_FFT = 2e-6
+TOL_V = 1e-6
+TOL_OP = TOL_FFT + TOL_V
+
+
+@pytest.fixture(scope="module")
+def nf():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1710_03197_gb300 as nf
+    return nf
+
+
+def rel(a, b):
+    return float(np.linalg.norm(np.ravel(a) - np.ravel(b)) / np.linalg.norm(b))
+
+
+def cn(shape, seed):
+    rng = np.random.default_rng(seed)
+    return (rng.standard_normal(shape) + 1j * rng.standard_normal(shape)).astype(np.complex64)
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+# (grid, image): axis-0 lines of 128 and 256 above and below the threshold for sixteen
+# values per thread, columns that 16 or 8 do not divide, the axis-1 pass with outer
+# lines, and images that fill more or less than half of the grid
+@pytest.mark.parametrize("Kd,Nd", [
+    ((128, 96, 64), (64, 48, 32)), ((256, 48, 64), (200, 24, 32)), ((128, 64, 64), (64, 32, 32)),
+    ((64, 128, 128), (64, 64, 100)), ((64, 256, 64), (50, 128, 64)), ((128, 90, 90), (64, 60, 90)),
+    ((256, 50, 30), (128, 26, 30)), ((16, 32, 1024), (16, 20, 512)), ((512, 128), (256, 128)), ((1024, 36), (512, 18)),
+    ((64, 512), (34, 512)),
+])
+def test_fft_passes(nf, Kd, Nd):
+    d = len(Kd)
+    om = W.uniform_random_om(7, d, seed=3)
+    p = oracle.make_plan(om, Nd, Kd, (6,) * d)
+    x, z = cn(Nd, 1), cn(Kd, 2)
+    with nf.NufftPlan(dev(om), Nd, Kd, (6,) * d) as plan:
+        assert rel(plan.scale_pad_fft(dev(x)).cpu().numpy(), oracle.fft_forward(oracle.scale_pad(p, x))) < TOL_FFT
+        assert rel(plan.ifft_crop_rescale(dev(z)).cpu().numpy(), oracle.crop_rescale(p, oracle.fft_adjoint(z))) < TOL_FFT
+
+
+@pytest.mark.parametrize("J", [4, 5, 6, 7])
+@pytest.mark.parametrize("Kd,M", [((32, 32, 32), 1), ((32, 32, 32), 6001), ((20, 24, 36), 1279), ((16, 18, 50), 81)])
+def test_3d_interpolation_and_gridding(nf, J, Kd, M):
+    Nd = tuple(2 * (K // 4) for K in Kd)
+    om = W.uniform_random_om(M, 3, seed=M + J)
+    p = oracle.make_plan(om, Nd, Kd, (J,) * 3)
+    z, y = cn(Kd, 4), cn(M, 5)
+    with nf.NufftPlan(dev(om), Nd, Kd, (J,) * 3) as plan:
+        assert rel(plan.interp(dev(z)).cpu().numpy(), oracle.interp_V(p, z)) < TOL_V
+        assert rel(plan.gridding(dev(y)).cpu().numpy(), oracle.gridding_VH(p, y)) < TOL_V
+
+
+# chunks of few and of many points, CTA counts on both sides of the rule, odd tiles
+@pytest.mark.parametrize("Jd", [(4, 4), (5, 5), (6, 6), (7, 7), (5, 7), (6, 1)])
+@pytest.mark.parametrize("Kd,M,nb", [((256, 256), 3001, 20), ((256, 256), 17000, 2), ((90, 64), 700, 3),
+                                     ((360, 288), 9000, 11)])
+def test_2d_batches(nf, Jd, Kd, M, nb):
+    Nd = tuple(2 * (K // 4) for K in Kd)
+    om = W.uniform_random_om(M, 2, seed=M)
+    om[: M // 8] = 0.1 + 0.02 * om[: M // 8]     # a dense tile of several chunks
+    p = oracle.make_plan(om, Nd, Kd, Jd)
+    xs, ys = cn((nb,) + Nd, 6), cn((nb, M), 7)
+    with nf.NufftPlan(dev(om), Nd, Kd, Jd) as plan:
+        yb, xb = plan.forward_batch(dev(xs)).cpu().numpy(), plan.adjoint_batch(dev(ys)).cpu().numpy()
+        again = plan.adjoint_batch(dev(ys)).cpu().numpy()
+    np.testing.assert_array_equal(again, xb)
+    for b in {0, 1, nb - 1}:
+        assert rel(yb[b], oracle.forward(p, xs[b])) < TOL_OP
+        assert rel(xb[b], oracle.adjoint(p, ys[b])) < TOL_OP
