@@ -1088,16 +1088,14 @@ __device__ __forceinline__ void reduce_tile(const float2* __restrict__ tiles, co
   __syncthreads();   // shared scratch free for the caller
 }
 
-// CTA x reduces slice x % slices of tile x / slices (slices of blockDim/NG*CPT cells).
+// CTA x reduces tile x.
 template <int D, int CPT, int TF>
 __global__ void __launch_bounds__(1024)
 k_gridding_reduce(const float2* __restrict__ tiles_b, const int32_t* __restrict__ bin_chunk,
-                  float2* __restrict__ grid_b, const Geom g, const int NG, int64_t tbs, int64_t gbs, int slices) {
+                  float2* __restrict__ grid_b, const Geom g, const int NG, int64_t tbs, int64_t gbs) {
   extern __shared__ float2 part[];
-  const int bin = blockIdx.x / slices;
-  const int cbase = (blockIdx.x - bin * slices) * (blockDim.x / NG) * CPT;
   reduce_tile<D, CPT, TF>(tiles_b + (int64_t)blockIdx.y * tbs, bin_chunk, grid_b + (int64_t)blockIdx.y * gbs, g,
-                             NG, bin, part, cbase);
+                          NG, blockIdx.x, part);
 }
 
 
@@ -1291,22 +1289,94 @@ k_gridding_chunk_staged(const float2* __restrict__ y_b, float2* __restrict__ til
   for (int c = threadIdx.x; c < ncell; c += blockDim.x) out[c] = fix_value<2>(acc, ncell, c, cs);
 }
 
+// 3D: thread (r1, r2) of a tile sums kRed3Planes cells of its column, r0 = z0 ..
+// z0 + kRed3Planes - 1, so one address and one neighbour test serve the whole
+// column, its loads are all in flight together, and a warp of rows r1 >= J - 1
+// skips the neighbours below along axis 1 as one.  The sum runs over e, then
+// over the source bin's chunks, from zero, as in reduce_tile (the same values).
+// CTA x: tile x / nsl, slice x % nsl = (column block, z0).  Measured on the
+// 128^3 kooshball (4096 tiles of 16^3, 226 MB of partial tiles, 134 MB of grid):
+// 184 us with four cells per thread and a neighbour mask for each.
+constexpr int kRed3Planes = 8;
+constexpr int kRed3Threads = 256;
+
+__global__ void __launch_bounds__(kRed3Threads)
+k_gridding_reduce3d(const float2* __restrict__ tiles_b, const int32_t* __restrict__ bin_chunk,
+                    float2* __restrict__ grid_b, const Geom g, int64_t tbs, int64_t gbs, int nsl, int nz) {
+  const float2* __restrict__ tiles = tiles_b + (int64_t)blockIdx.y * tbs;
+  float2* __restrict__ grid = grid_b + (int64_t)blockIdx.y * gbs;
+  const int bin = blockIdx.x / nsl;
+  const int sl = blockIdx.x - bin * nsl;
+  const int z0 = (sl % nz) * kRed3Planes;
+  const int pos = (sl / nz) * blockDim.x + threadIdx.x;
+  const int b2 = bin % g.nb[2], b01 = bin / g.nb[2], b1 = b01 % g.nb[1], b0 = b01 / g.nb[1];
+  const int r1 = pos / g.T[2], r2 = pos - r1 * g.T[2];
+  if (r1 >= g.T[1]) return;   // no barriers below
+  const int plane = g.P[1] * g.P[2];
+  const int nzc = min(kRed3Planes, g.T[0] - z0);   // cells of the column here
+  float2 acc[kRed3Planes];
+#pragma unroll
+  for (int k = 0; k < kRed3Planes; ++k) acc[k] = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const int e0 = e >> 2, e1 = (e >> 1) & 1, e2 = e & 1;
+    const int n = e0 ? min(nzc, g.J[0] - 1 - z0) : nzc;   // the neighbour below reaches r0 < J - 1
+    if (n <= 0 || (e1 && r1 >= g.J[1] - 1) || (e2 && r2 >= g.J[2] - 1)) continue;
+    const int s0 = e0 ? (b0 > 0 ? b0 : g.nb[0]) - 1 : b0;
+    const int s1 = e1 ? (b1 > 0 ? b1 : g.nb[1]) - 1 : b1;
+    const int s2 = e2 ? (b2 > 0 ? b2 : g.nb[2]) - 1 : b2;
+    const int src = (s0 * g.nb[1] + s1) * g.nb[2] + s2;
+    const int q1 = __ldg(&bin_chunk[src + 1]);
+    int q = __ldg(&bin_chunk[src]);
+    const float2* ptr = tiles + (int64_t)q * g.padded_cells +
+                        ((z0 + e0 * g.T[0]) * g.P[1] + r1 + e1 * g.T[1]) * g.P[2] + r2 + e2 * g.T[2];
+    if (n == kRed3Planes) {
+      for (; q < q1; ++q, ptr += g.padded_cells) {
+        float2 v[kRed3Planes];
+#pragma unroll
+        for (int k = 0; k < kRed3Planes; ++k) v[k] = __ldg(&ptr[k * plane]);
+#pragma unroll
+        for (int k = 0; k < kRed3Planes; ++k) acc[k] = cadd(acc[k], v[k]);
+      }
+    } else {
+      for (; q < q1; ++q, ptr += g.padded_cells) {
+        float2 v[kRed3Planes];
+#pragma unroll
+        for (int k = 0; k < kRed3Planes; ++k) v[k] = k < n ? __ldg(&ptr[k * plane]) : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < kRed3Planes; ++k)
+          if (k < n) acc[k] = cadd(acc[k], v[k]);
+      }
+    }
+  }
+  float2* out = grid + ((b0 * g.T[0] + z0) * (int)g.Kstride[0] + (b1 * g.T[1] + r1) * (int)g.Kstride[1] +
+                        b2 * g.T[2] + r2);
+#pragma unroll
+  for (int k = 0; k < kRed3Planes; ++k)
+    if (k < nzc) out[k * (int)g.Kstride[0]] = acc[k];
+}
+
 // The reduction gives every thread 4 cells of the tile; small tiles get up to 4
 // thread groups, each summing every 4th (neighbour, chunk) pair.
 template <int D>
 cudaError_t launch_reduce(const nufft_plan_t* p, const float2* tiles, float2* grid, int nb = 1) {
+  if constexpr (D == 3) {
+    const Geom& g = p->g;
+    const int cols = g.T[1] * g.T[2];
+    const int threads = std::min(kRed3Threads, (cols + 31) / 32 * 32);
+    const int nz = (g.T[0] + kRed3Planes - 1) / kRed3Planes;
+    const int nsl = nz * ((cols + threads - 1) / threads);
+    k_gridding_reduce3d<<<dim3((unsigned)(g.nbins * nsl), (unsigned)nb), threads, 0, p->stream>>>(
+        tiles, p->bin_chunk, grid, g, p->nchunks * g.padded_cells, p->Kprod, nsl, nz);
+    return cudaGetLastError();
+  }
   int cells = 1;
   for (int a = 0; a < D; ++a) cells *= p->g.T[a];
-  // 3D 16^3 tiles: an eighth of a tile (512 cells) per CTA of 128 threads, so
-  // that many tiles' set-up, loads and stores overlap on an SM (one 1024-thread
-  // CTA of 64 registers filled an SM: 1 -> 2 -> 4 -> 8 slices measured 0.909,
-  // 0.887, 0.875, 0.864 ms for the kooshball's gridding; 16 no better)
-  const int slices = (D == 3 && cells >= 4096) ? 8 : 1;
-  const int gsize = std::max(32, std::min(1024, (cells / slices + 4 * 32 - 1) / (4 * 32) * 32));
-  if ((int64_t)gsize * 4 * slices < cells) return cudaErrorInvalidValue;
+  const int gsize = std::max(32, std::min(1024, (cells + 4 * 32 - 1) / (4 * 32) * 32));
+  if ((int64_t)gsize * 4 < cells) return cudaErrorInvalidValue;
   // groups splitting the chunk list; a batch (mostly sparse tiles, many CTAs)
   // runs one group per CTA so that more tiles are in flight per SM
-  const int NG = (nb > 1 || slices > 1) ? 1 : std::max(1, std::min(4, 1024 / gsize));
+  const int NG = nb > 1 ? 1 : std::max(1, std::min(4, 1024 / gsize));
   const size_t smem = NG > 1 ? (size_t)NG * 4 * gsize * sizeof(float2) : 0;
   bool t16 = D > 1;
   for (int a = 0; a < D; ++a) t16 = t16 && p->g.T[a] == 16;
@@ -1320,9 +1390,11 @@ cudaError_t launch_reduce(const nufft_plan_t* p, const float2* tiles, float2* gr
       return cudaGetLastError();
     }
   }
-  auto kern = t16 ? k_gridding_reduce<D, 4, (D > 1 ? 16 : 0)> : k_gridding_reduce<D, 4, 0>;
-  kern<<<dim3((unsigned)(p->g.nbins * slices), (unsigned)nb), gsize * NG, smem, p->stream>>>(
-      tiles, p->bin_chunk, grid, p->g, NG, p->nchunks * p->g.padded_cells, p->Kprod, slices);
+  if constexpr (D < 3) {
+    auto kern = t16 ? k_gridding_reduce<D, 4, (D > 1 ? 16 : 0)> : k_gridding_reduce<D, 4, 0>;
+    kern<<<dim3((unsigned)p->g.nbins, (unsigned)nb), gsize * NG, smem, p->stream>>>(
+        tiles, p->bin_chunk, grid, p->g, NG, p->nchunks * p->g.padded_cells, p->Kprod);
+  }
   return cudaGetLastError();
 }
 
