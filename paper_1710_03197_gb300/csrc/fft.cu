@@ -17,12 +17,12 @@
 // Padded position of image index n along an axis: g = (n - N/2) mod K.
 //
 // Each line of power-of-two length is transformed by a Stockham auto-sort
-// FFT (one radix-2 or radix-4 stage, then radix-8 stages), each thread
-// holding 8 values per stage in registers.  The first stage works on the values as loaded and
-// the last stage's outputs are stored as they are; the hand-offs between
-// stages go through two shared-memory buffers used in turn, one barrier per
-// hand-off.  Twiddles exp(-2 pi i k / K) come from a table computed in FP64 at
-// plan time and are loaded before the barrier of the stage that uses them.
+// FFT, each thread holding E values per stage in registers: one smaller radix
+// if the length asks for it, then radix-E stages, E = 8 or 16.  The first stage
+// works on the values as loaded and the last stage's outputs are stored as they
+// are; the hand-offs between stages go through two shared-memory buffers used
+// in turn (one buffer where there is one hand-off), one barrier per hand-off.
+// Twiddles are computed in registers.
 // Other line lengths (even, prime factors 2, 3 and 5) run a Stockham FFT of
 // radix-8, -4/-2, -3 and -5 stages through shared memory (k_fft_mixed).
 #include "internal.cuh"
@@ -136,160 +136,227 @@ __device__ __forceinline__ void dft8(float2* v) {
   v[3] = cadd(e3, o3); v[7] = csub(e3, o3);
 }
 
+// DFT of 16 points as 4 x 4: DFT-4 over (i, i + 4, i + 8, i + 12), twiddles
+// W16^(i j), DFT-4 over i.
+template <bool INV>
+__device__ __forceinline__ void dft16(float2* v) {
+  const float h = 0.70710678118654752440f, c = 0.92387953251128675613f, s = 0.38268343236508977173f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) dft4<INV>(v[i], v[i + 4], v[i + 8], v[i + 12]);
+  // v[i + 4 j] *= W16^(i j), W16 = exp(-+ 2 pi i / 16) = c -+ i s
+  auto mul = [](float2 z, float wr, float wi) { return cmul(z, make_float2(wr, INV ? -wi : wi)); };
+  v[5] = mul(v[5], c, -s);
+  v[9] = INV ? make_float2(h * (v[9].x - v[9].y), h * (v[9].x + v[9].y))
+             : make_float2(h * (v[9].x + v[9].y), h * (v[9].y - v[9].x));
+  v[13] = mul(v[13], s, -c);
+  v[6] = INV ? make_float2(h * (v[6].x - v[6].y), h * (v[6].x + v[6].y))
+             : make_float2(h * (v[6].x + v[6].y), h * (v[6].y - v[6].x));
+  v[10] = rot90<INV>(v[10]);
+  v[14] = INV ? make_float2(h * (-v[14].x - v[14].y), h * (v[14].x - v[14].y))
+              : make_float2(h * (v[14].y - v[14].x), h * (-v[14].x - v[14].y));
+  v[7] = mul(v[7], s, -c);
+  v[11] = INV ? make_float2(h * (-v[11].x - v[11].y), h * (v[11].x - v[11].y))
+              : make_float2(h * (v[11].y - v[11].x), h * (-v[11].x - v[11].y));
+  v[15] = mul(v[15], -c, s);
+  float2 o[16];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    dft4<INV>(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) o[j + 4 * q] = v[4 * j + q];   // output j + 4 q
+  }
+#pragma unroll
+  for (int k = 0; k < 16; ++k) v[k] = o[k];
+}
+
 template <int R, bool INV>
 __device__ __forceinline__ void dft(float2* v) {
   if (R == 2) dft2<INV>(v);
   else if (R == 4) dft4<INV>(v[0], v[1], v[2], v[3]);
-  else dft8<INV>(v);
+  else if (R == 8) dft8<INV>(v);
+  else dft16<INV>(v);
 }
 
 constexpr int ilog2(int x) { return x <= 1 ? 0 : 1 + ilog2(x / 2); }
 
-// Shared-memory position of element p of the line owned by lane-group b.
-// Contiguous axis: one line after another, one pad word per 8 elements.
-// Strided axis: W lines side by side (W consecutive grid columns), row pitch W+1.
+// Shared-memory position of element p of line b of the CTA's W lines, for the
+// hand-off after a stage of radix R and span Ns.  A half-warp's 64-bit accesses
+// are free of conflicts when its 16 positions differ mod 16.
+// Strided axis: W lines side by side (W consecutive grid columns), a row of W
+// values per element: 16 columns fill a half-warp; with fewer, the writers of
+// the first hand-off (Ns = 1, row stride R from one thread to the next) need
+// the row's low bits mixed with the thread's.
+// Contiguous axis: one line after another, one pad word per 16 elements (8 in
+// lines of at most 128), and a pitch of 8 mod 16 for lines whose 8 threads
+// share a half-warp with the next line's.
 template <int L, bool STRIDED>
 struct SmemMap {
-  int w;  // lines per CTA
-  static constexpr int kLinePitch = L + L / 8;
-  __device__ __forceinline__ int at(int b, int p) const {
-    return STRIDED ? p * (w + 1) + b : b * kLinePitch + p + (p >> 3);
+  static constexpr int kPad = L <= 128 ? 3 : 4;
+  static constexpr int kRaw = L + (L >> kPad);
+  static constexpr int kLinePitch = L == 128 ? 152 : kRaw;
+  template <int R, int NS>
+  __device__ __forceinline__ static int at(int wlog, int b, int p) {
+    if (!STRIDED) return b * kLinePitch + p + (p >> kPad);
+    const int q = NS == 1 && wlog < 4 ? p ^ ((p / R) & ((16 >> wlog) - 1)) : p;
+    return (q << wlog) + b;
   }
-  __host__ __device__ static size_t words(int w) { return STRIDED ? (size_t)L * (w + 1) : (size_t)w * kLinePitch; }
+  __host__ __device__ static size_t words(int w) { return STRIDED ? (size_t)L * w : (size_t)w * kLinePitch; }
 };
 
 // Stockham stage of radix R over span Ns on the values a thread holds.
 //
-// In every stage a thread reads the elements t + k*TPL (k = 0..7) of its line:
-// butterfly q (q < 8/R) takes inputs j + r*L/R with j = t + q*TPL, which is
-// element t + (q + r*Q)*TPL.  So x[k] holds element t + k*TPL on entry, the
-// first stage needs no shared memory, and the outputs of the last stage
+// In every stage a thread reads the elements t + k*TPL (k = 0..E-1, TPL = L/E)
+// of its line: butterfly q (q < E/R) takes inputs j + r*L/R with j = t + q*TPL,
+// which is element t + (q + r*Q)*TPL.  So x[k] holds element t + k*TPL on entry,
+// the first stage needs no shared memory, and the outputs of the last stage
 // (Ns = L/R, written to j + r*Ns) are again elements t + k*TPL, stored straight
 // to global memory.  Only the middle hand-offs go through shared memory.
-template <int L, int R>
-struct StageTw {                      // twiddles of one stage
-  float2 w[8 / R][R];
-};
-
-// Twiddles of a radix-8 stage, computed: input r of the thread's butterfly
-// gets w1^r, w1 = exp(-+ 2 pi i k / (Ns R)), from sincospif (2k / (Ns R) is
-// exact: Ns R is a power of two) and products of depth at most three (a few
-// ulp; a table rounded from FP64 would be 0.5 ulp).  The passes then issue no
-// twiddle loads (the strided 3D passes are bound by the L1/shared pipe, the
-// 2D ones by load latency).
-template <int L, bool INV>
-__device__ __forceinline__ void make_twiddles8(StageTw<L, 8>& T, int t, int Ns) {
-  const float inv = 2.0f / (float)(Ns * 8);   // exact
-  const int k = t & (Ns - 1);                  // radix 8: one butterfly per thread
+//
+// Twiddles of a radix-E stage, computed: input r of the thread's butterfly gets
+// w1^r, w1 = exp(-+ 2 pi i k / (Ns E)), from sincospif (2k / (Ns E) is exact:
+// Ns E is a power of two) and products (a few ulp; a table rounded from FP64
+// would be 0.5 ulp).  Radix 16 takes w4 from sincospif too, so that no power
+// carries more than six single errors.  The passes then issue no twiddle loads
+// (the strided 3D passes are bound by issue and the L1/shared pipe, the 2D ones
+// by load latency).
+template <int E, bool INV>
+__device__ __forceinline__ void apply_twiddles(float2 (&x)[E], int k, int Ns) {
+  const float inv = 2.0f / (float)(Ns * E);   // exact
   float sn, cs;
   sincospif((float)k * inv, &sn, &cs);
   const float2 w1 = make_float2(cs, INV ? sn : -sn);
-  const float2 w2 = cmul(w1, w1), w4 = cmul(w2, w2);
-  T.w[0][1] = w1;
-  T.w[0][2] = w2;
-  T.w[0][3] = cmul(w2, w1);
-  T.w[0][4] = w4;
-  T.w[0][5] = cmul(w4, w1);
-  T.w[0][6] = cmul(w4, w2);
-  T.w[0][7] = cmul(w4, T.w[0][3]);
+  const float2 w2 = cmul(w1, w1), w3 = cmul(w2, w1);
+  float2 w4;
+  if (E == 16) {
+    sincospif((float)(4 * k) * inv, &sn, &cs);
+    w4 = make_float2(cs, INV ? sn : -sn);
+  } else {
+    w4 = cmul(w2, w2);
+  }
+  float2 hi = w4;
+  x[1] = cmul(x[1], w1);
+  x[2] = cmul(x[2], w2);
+  x[3] = cmul(x[3], w3);
+#pragma unroll
+  for (int r = 4; r < E; r += 4) {
+    x[r] = cmul(x[r], hi);
+    x[r + 1] = cmul(x[r + 1], cmul(hi, w1));
+    x[r + 2] = cmul(x[r + 2], cmul(hi, w2));
+    x[r + 3] = cmul(x[r + 3], cmul(hi, w3));
+    if (r + 4 < E) hi = cmul(hi, w4);
+  }
 }
 
-template <int L, bool INV, int R, bool TW>
-__device__ __forceinline__ void butterflies(float2 (&x)[8], const StageTw<L, R>& T) {
-  constexpr int Q = 8 / R;
+template <int E, int R, bool INV>
+__device__ __forceinline__ void butterflies(float2 (&x)[E]) {
+  constexpr int Q = E / R;
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     float2 v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = x[q + r * Q];
-    if (TW) {
-#pragma unroll
-      for (int r = 1; r < R; ++r) v[r] = cmul(v[r], T.w[q][r]);
-    }
     dft<R, INV>(v);
 #pragma unroll
     for (int r = 0; r < R; ++r) x[q + r * Q] = v[r];
   }
 }
 
-// Write the outputs of a stage (radix R, span Ns) to their Stockham positions.
-template <int L, bool STRIDED, int R>
-__device__ __forceinline__ void write_stage(float2* sm, const SmemMap<L, STRIDED> SI, int b, int t, int Ns,
-                                            const float2 (&x)[8]) {
-  constexpr int TPL = L / 8;
-  constexpr int Q = 8 / R;
+// Hand-off after a stage of radix R and span NS: outputs to their Stockham
+// positions, barrier, the thread's next elements.
+template <int L, int E, bool STRIDED, int R, int NS>
+__device__ __forceinline__ void hand_off(float2* sm, int wlog, int b, int t, float2 (&x)[E]) {
+  constexpr int TPL = L / E;
+  constexpr int Q = E / R;
+  using Map = SmemMap<L, STRIDED>;
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     const int j = t + q * TPL;
-    const int k = j & (Ns - 1);
+    const int k = j & (NS - 1);
     const int base = (j - k) * R + k;
 #pragma unroll
-    for (int r = 0; r < R; ++r) sm[SI.at(b, base + r * Ns)] = x[q + r * Q];
+    for (int r = 0; r < R; ++r) sm[Map::template at<R, NS>(wlog, b, base + r * NS)] = x[q + r * Q];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < E; ++k) x[k] = sm[Map::template at<R, NS>(wlog, b, t + k * TPL)];
+}
+
+// Stages of radix E from span NS on; buffer c of the two at sm + c * bufw.
+template <int L, int E, bool STRIDED, bool INV, int NS>
+__device__ __forceinline__ void radix_e_stages(float2* sm, int cur, int bufw, int wlog, int b, int t, float2 (&x)[E]) {
+  if (NS > 1) apply_twiddles<E, INV>(x, t & (NS - 1), NS);
+  butterflies<E, E, INV>(x);
+  if constexpr (NS * E < L) {
+    hand_off<L, E, STRIDED, E, NS>(sm + cur * bufw, wlog, b, t, x);
+    radix_e_stages<L, E, STRIDED, INV, NS * E>(sm, cur ^ 1, bufw, wlog, b, t, x);
   }
 }
 
-template <int L, bool STRIDED>
-__device__ __forceinline__ void read_own(const float2* sm, const SmemMap<L, STRIDED> SI, int b, int t,
-                                         float2 (&x)[8]) {
-  constexpr int TPL = L / 8;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) x[k] = sm[SI.at(b, t + k * TPL)];
-}
+constexpr int fft_first_radix(int L, int E) { return 1 << (ilog2(L) % ilog2(E)); }
+constexpr int fft_hand_offs(int L, int E) { return (ilog2(L) + ilog2(E) - 1) / ilog2(E) - 1; }
 
-template <int L, bool STRIDED, bool INV>
-__global__ void __launch_bounds__(STRIDED ? L : 256)
-k_fft_pass(const FftArgs A, const int W) {
-  constexpr int TPL = L / 8;
-  const SmemMap<L, STRIDED> SI{W};
+// grid: strided axes (column blocks, outer lines, batch), contiguous axis
+// (blocks of W lines, 1, batch); 32-bit indices within a transform (K^d <= 2^30).
+// HOOK: the CG step's work (contiguous axis only); a kernel of its own, so that
+// the plain pass carries none of its FP64 code.
+// WL > 0: log2 of the columns per CTA, fixed, so that the shared-memory addresses
+// of a hand-off are one base and immediate offsets; WL = 0: wl_arg.
+template <int L, int E, bool STRIDED, bool INV, bool HOOK, int WL>
+__global__ void __launch_bounds__(E == 16 ? 256 : (STRIDED ? L : 256), E == 16 ? 4 : 1)
+k_fft_pass(const FftArgs A, const int wl_arg) {
+  constexpr int TPL = L / E;
+  const int wlog = WL > 0 ? WL : wl_arg;
   extern __shared__ float2 sm[];
-  const int bufw = (int)SmemMap<L, STRIDED>::words(W);   // buffer c at sm + c * bufw
+  const int W = 1 << wlog;
+  const int bufw = (int)SmemMap<L, STRIDED>::words(W);
 
   const int tid = threadIdx.x;
-  int b, t;
-  int64_t o, in;
+  int b, t, o, in;
   if (STRIDED) {
-    b = tid % W;
-    t = tid / W;
-    const int64_t nib = A.inner / W;
-    o = blockIdx.x / nib;
-    in = (blockIdx.x % nib) * W + b;
+    b = tid & (W - 1);
+    t = tid >> wlog;
+    o = blockIdx.y;
+    in = blockIdx.x * W + b;
   } else {
     b = tid / TPL;
     t = tid % TPL;
-    o = (int64_t)blockIdx.x * W + b;
+    o = blockIdx.x * W + b;
     in = 0;
   }
-  const bool live = o < A.nouter;
-  const float2* __restrict__ src = A.src + (int64_t)blockIdx.y * A.src_bstride;
-  float2* __restrict__ dst = A.dst + (int64_t)blockIdx.y * A.dst_bstride;
+  const bool live = o < (int)A.nouter;
+  const float2* __restrict__ src = A.src + (int64_t)blockIdx.z * A.src_bstride;
+  float2* __restrict__ dst = A.dst + (int64_t)blockIdx.z * A.dst_bstride;
 
   // Outer coordinates: image index on axes < a, mapped to padded grid positions.
-  int64_t goff = 0;
+  int goff = in;
   float slead = 1.0f;
   if (live) {
-    int64_t rem = o;
+    int rem = o;
     for (int i = A.a - 1; i >= 0; --i) {
-      const int n = (int)(rem % A.lead_N[i]);
-      rem /= A.lead_N[i];
+      int n = rem;
+      if (i > 0) {   // the outermost coordinate is what is left
+        rem = n / A.lead_N[i];
+        n -= rem * A.lead_N[i];
+      }
       const int gi = wrapk(n - A.lead_N[i] / 2 + A.lead_K[i], A.lead_K[i]);
-      goff += (int64_t)gi * A.lead_stride[i];
+      goff += gi * (int)A.lead_stride[i];
       if (A.scale && (A.src_image || A.dst_image)) slead *= A.s_lead[i][n];
     }
   }
   const int half = A.Na >> 1;
-  const int64_t stride = A.inner;
-  __shared__ double red[32];
-  const bool pro = !INV && A.src_image && A.pro_p;
-  const float beta = pro ? cg_prologue_beta(A, red) : 0.f;
+  const int stride = STRIDED ? (int)A.inner : 1;
+  const bool pro = HOOK && !INV && A.src_image && A.pro_p;
+  float beta = 0.f;
+  if constexpr (HOOK && !INV) {
+    __shared__ double red[32];
+    if (pro) beta = cg_prologue_beta(A, red);
+  }
   const uint64_t pol = l2_evict_first_policy();   // a pass reads each input element once
 
-  constexpr int LOG = ilog2(L);
-  constexpr int R0 = 1 << (LOG % 3);
-  constexpr int N8 = LOG / 3;
   // ---- load the thread's elements t + k*TPL (pruned on the forward side)
-  float2 x[8];
+  float2 x[E];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
+  for (int k = 0; k < E; ++k) {
     const int p = t + k * TPL;
     float2 v = make_float2(0.f, 0.f);
     if (live) {
@@ -300,55 +367,36 @@ k_fft_pass(const FftArgs A, const int W) {
             const int n = p < half ? p + half : p - L + half;
             v = cscale(load_image(A, src, o * A.Na + n, pro, beta), (A.scale ? A.s_axis[n] : 1.0f) * slead);
           } else {
-            v = ld_last_use(&src[goff + (int64_t)p * stride + in], pol);
+            v = ld_last_use(&src[goff + p * stride], pol);
           }
         }
       } else {
-        v = ld_last_use(&src[goff + (int64_t)p * stride + in], pol);
+        v = ld_last_use(&src[goff + p * stride], pol);
       }
     }
     x[k] = v;
   }
 
-  // ---- transform: an optional radix-2/4 stage, then radix-8 stages
-  int Ns = 1;
-  int cur = 0;
-  if (R0 > 1) {
-    StageTw<L, R0> none;
-    butterflies<L, INV, R0, false>(x, none);
-    write_stage<L, STRIDED, R0>(sm, SI, b, t, 1, x);
-    Ns = R0;
-  }
-#pragma unroll
-  for (int s = 0; s < N8; ++s) {
-    StageTw<L, 8> T;
-    const bool first = (R0 == 1 && s == 0);
-    if (!first) {
-      make_twiddles8<L, INV>(T, t, Ns);
-      __syncthreads();
-      read_own<L, STRIDED>(sm + cur * bufw, SI, b, t, x);
-      butterflies<L, INV, 8, true>(x, T);
-    } else {
-      butterflies<L, INV, 8, false>(x, T);
-    }
-    if (s + 1 < N8) {
-      const int nxt = first ? 0 : cur ^ 1;
-      write_stage<L, STRIDED, 8>(sm + nxt * bufw, SI, b, t, Ns, x);
-      cur = nxt;
-    }
-    Ns *= 8;
+  // ---- transform: a smaller first radix where the length needs one, then radix E
+  constexpr int R0 = fft_first_radix(L, E);
+  if constexpr (R0 > 1) {
+    butterflies<E, R0, INV>(x);
+    hand_off<L, E, STRIDED, R0, 1>(sm, wlog, b, t, x);
+    radix_e_stages<L, E, STRIDED, INV, R0>(sm, 1, bufw, wlog, b, t, x);
+  } else {
+    radix_e_stages<L, E, STRIDED, INV, 1>(sm, 0, bufw, wlog, b, t, x);
   }
 
   // ---- store the thread's elements t + k*TPL (pruned on the inverse side)
-  const bool epi = INV && A.dst_image && A.epi_part;
+  const bool epi = HOOK && INV && A.dst_image && A.epi_part;
   double dot = 0.0;
   if (live) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
+    for (int k = 0; k < E; ++k) {
       const int p = t + k * TPL;
       const float2 v = x[k];
       if (!INV) {
-        dst[goff + (int64_t)p * stride + in] = v;
+        dst[goff + p * stride] = v;
       } else {
         const bool in_image = (p < half) || (p >= L - half);
         if (!in_image) continue;
@@ -361,53 +409,84 @@ k_fft_pass(const FftArgs A, const int W) {
             dot += (double)a.x * (double)out.x + (double)a.y * (double)out.y;
           }
         } else {
-          dst[goff + (int64_t)p * stride + in] = v;
+          dst[goff + p * stride] = v;
         }
       }
     }
   }
-  if (epi) {
-    const double tsum = block_sum_dbl(dot, red);
-    if (threadIdx.x == 0) A.epi_part[blockIdx.x] = tsum;
+  if constexpr (HOOK && INV) {
+    __shared__ double red[32];
+    if (epi) {
+      const double tsum = block_sum_dbl(dot, red);
+      if (threadIdx.x == 0) A.epi_part[blockIdx.x] = tsum;
+    }
   }
 }
 
-// Lines per CTA: as many as give 256 threads (8 columns on a strided axis, for
-// 64-byte row segments), fewer when that would leave the GPU with fewer than
-// two CTAs per SM (counting every batch element's CTAs).
+// CTAs wanted before lines are grouped into wider ones.
 constexpr int64_t kTargetBlocks = 2 * 152;
 
 // query: only report the number of CTAs (per batch element) in *nblocks.
-template <int L, bool STRIDED, bool INV>
-cudaError_t launch_L(const FftArgs& A, int nb, cudaStream_t st, int64_t* nblocks, bool query) {
-  constexpr int TPL = L / 8;
-  int W;
+// E values per thread.  Lines per CTA: as many as give 256 threads (strided
+// axis: at most 16 columns, full 128-byte rows with E = 16, 8 with E = 8), fewer
+// when that would leave the GPU with fewer than two CTAs per SM (counting every
+// batch element's CTAs).
+template <int L, int E, bool STRIDED, bool INV>
+cudaError_t launch_LE(const FftArgs& A, int nb, cudaStream_t st, int64_t* nblocks, bool query) {
+  constexpr int TPL = L / E;
+  constexpr int kBuffers = fft_hand_offs(L, E) > 1 ? 2 : 1;
+  int wlog = 0;
   int64_t blocks;
   if (STRIDED) {
-    W = 8;
-    while (W > 2 && (A.inner % W != 0 || A.nouter * (A.inner / W) * nb < kTargetBlocks ||
-                     2 * SmemMap<L, STRIDED>::words(W) * sizeof(float2) > 96 * 1024))
-      W >>= 1;
-    blocks = A.nouter * (A.inner / W);
+    wlog = E == 16 ? std::min(4, ilog2(256 / TPL)) : 3;
+    while (wlog > 1 && (A.inner % (1 << wlog) != 0 || A.nouter * (A.inner >> wlog) * nb < kTargetBlocks ||
+                        kBuffers * SmemMap<L, STRIDED>::words(1 << wlog) * sizeof(float2) > 96 * 1024))
+      --wlog;
+    blocks = A.nouter * (A.inner >> wlog);
   } else {
-    W = TPL >= 256 ? 1 : 256 / TPL;
-    while (W > 1 && (A.nouter + W - 1) / W * nb < kTargetBlocks) W >>= 1;
-    blocks = (A.nouter + W - 1) / W;
+    wlog = TPL >= 256 ? 0 : ilog2(256 / TPL);
+    while (wlog > 0 && ((A.nouter + (1 << wlog) - 1) >> wlog) * nb < kTargetBlocks) --wlog;
+    blocks = (A.nouter + (1 << wlog) - 1) >> wlog;
   }
   if (nblocks) *nblocks = blocks;
   if (query) return cudaSuccess;
-  const int threads = W * TPL;
-  const size_t smem = 2 * SmemMap<L, STRIDED>::words(W) * sizeof(float2);   // ping-pong buffers
-  // always: the kernel's static shared memory (the CG hooks' scratch) comes on
-  // top, so even a 48 KB request needs the opt-in
-  cudaError_t e = cudaFuncSetAttribute(k_fft_pass<L, STRIDED, INV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return e;
-  if (blocks == 0) return cudaSuccess;
-  k_fft_pass<L, STRIDED, INV><<<dim3((unsigned)blocks, (unsigned)nb), threads, smem, st>>>(A, W);
-  return cudaGetLastError();
+  const size_t smem = kBuffers * SmemMap<L, STRIDED>::words(1 << wlog) * sizeof(float2);
+  auto go = [&](auto kern) {
+    // always: static shared memory (the CG hooks' scratch) comes on top, so even
+    // a 48 KB request needs the opt-in
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess || blocks == 0) return e;
+    const dim3 gd = STRIDED ? dim3((unsigned)(A.inner >> wlog), (unsigned)A.nouter, (unsigned)nb)
+                            : dim3((unsigned)blocks, 1, (unsigned)nb);
+    kern<<<gd, TPL << wlog, smem, st>>>(A, wlog);
+    return cudaGetLastError();
+  };
+  if constexpr (!STRIDED) {
+    if (A.pro_p || A.epi_part) return go(k_fft_pass<L, E, STRIDED, INV, true, 0>);
+  } else {
+    constexpr int kFull = E == 16 ? 4 : 3;
+    if (wlog == kFull) return go(k_fft_pass<L, E, STRIDED, INV, false, kFull>);
+  }
+  return go(k_fft_pass<L, E, STRIDED, INV, false, 0>);
 }
 
+// Sixteen values per thread on strided axes of 128 and 256 points that still
+// fill the GPU: one hand-off instead of two, fewer twiddles per value, and
+// 128-byte rows (on a 256^3 grid's passes 30 -> 28 us and 54 -> 50 us forward,
+// 57 -> 43 us and 29 -> 24 us inverse against eight).  Longer lines need two
+// hand-offs either way and lose to the registers (32 transforms of 512^2: 35 us
+// against 30), the contiguous passes to them and to the scaling's loads, and a
+// small pass is bound by latency: all these take eight, with twice the warps.
+constexpr int64_t kWideWarps = 8 * 152;
+
+template <int L, bool STRIDED, bool INV>
+cudaError_t launch_L(const FftArgs& A, int nb, cudaStream_t st, int64_t* nblocks, bool query) {
+  if constexpr (STRIDED && (L == 128 || L == 256)) {
+    if (A.nouter * A.inner * nb * (L / 16) >= kWideWarps * 32 && A.inner % 16 == 0)
+      return launch_LE<L, 16, STRIDED, INV>(A, nb, st, nblocks, query);
+  }
+  return launch_LE<L, 8, STRIDED, INV>(A, nb, st, nblocks, query);
+}
 
 // ---------------------------------------------------------------- other line lengths
 // Stockham FFT of a line of length L = 2^a 3^b 5^c through shared memory:
