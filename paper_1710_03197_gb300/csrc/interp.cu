@@ -55,6 +55,51 @@ __device__ __forceinline__ float2 lane_group_sum(float2 part, int base, int G) {
   }
 }
 
+// 2D batches: a thread takes kBatchPer batch elements in turn with the point's
+// neighbours and coefficients in registers (JF > 0), so that each element costs
+// its J_0 grid loads only.
+constexpr int kBatchPer = 4;
+
+template <int JF>
+__global__ void __launch_bounds__(256)
+k_interp_batch2d(const float2* __restrict__ grid_b, float2* __restrict__ y_b, const Points P, const Geom g, int64_t gbs,
+                 int64_t ybs, int nb) {
+  const int lane = threadIdx.x & 31;
+  constexpr int PW = 32 / JF;
+  const int sub = lane / JF;
+  const int l = lane - sub * JF;
+  const int64_t i = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * PW + sub;
+  const bool active = sub < PW && i < P.M;
+  float2 c0[JF], cl = make_float2(0.f, 0.f);
+  int off[JF], m = 0;
+#pragma unroll
+  for (int j = 0; j < JF; ++j) {
+    c0[j] = make_float2(0.f, 0.f);
+    off[j] = 0;
+  }
+  if (active) {
+    const int k0 = P.kf[i];
+    const int gl = wrapk(P.kf[P.M + i] + l, g.K[1]);
+    m = P.perm[i];
+    cl = P.coef[P.coef_off[1] + (int64_t)l * P.M + i];
+#pragma unroll
+    for (int j = 0; j < JF; ++j) {
+      c0[j] = P.coef[P.coef_off[0] + (int64_t)j * P.M + i];
+      off[j] = wrapk(k0 + j, g.K[0]) * (int)g.Kstride[0] + gl;
+    }
+  }
+  const int b0 = blockIdx.y * kBatchPer, b1 = min(nb, b0 + kBatchPer);
+  const float2* __restrict__ grid = grid_b + b0 * gbs;
+  float2* __restrict__ y = y_b + b0 * ybs + m;
+  for (int b = b0; b < b1; ++b, grid += gbs, y += ybs) {   // CTA-uniform
+    float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < JF; ++j) acc = cfma(c0[j], __ldg(&grid[off[j]]), acc);
+    const float2 tot = lane_group_sum<JF>(cmul(cl, acc), sub * JF, JF);
+    if (active && l == 0) *y = tot;
+  }
+}
+
 template <int D, int JF>
 __global__ void __launch_bounds__(256)
 k_interp(const float2* __restrict__ grid_b, float2* __restrict__ y_b, const Points P, const Geom g, int64_t gbs,
@@ -1289,6 +1334,192 @@ k_gridding_chunk_staged(const float2* __restrict__ y_b, float2* __restrict__ til
   for (int c = threadIdx.x; c < ncell; c += blockDim.x) out[c] = fix_value<2>(acc, ncell, c, cs);
 }
 
+// ---------------------------------------------------------------- 2D chunk passes of a batch
+// V and V^H of one chunk of a 2D tile for one batch element, per CTA of two
+// warps.  A batch has CTAs enough, and the chunks of a dynamic series' frames are
+// small (30 points), so what counts is the instructions spent per CTA: eight
+// warps with staged point data (k_gridding_chunk_staged) spend most of theirs on
+// set-up, barriers and idle warps.  A single transform keeps that kernel: its
+// few CTAs are bound by latency, which staging everything at once hides better
+// (a 512^2 grid with 206,336 points: 56 us for the pair, 67 us with these).
+// The lane
+// layout is that of k_interp (a group of J_1 lanes per point, lane l its l-th
+// neighbour along the contiguous axis); every warp loads the next round's point
+// data into registers while it works on this one's (no barrier between rounds):
+// lane l of a point loads c_0[l] and c_1[l], keeps c_1[l] for its own column and
+// passes c_0[l] to the point's other lanes through a per-warp strip of shared
+// memory.  JF > 0: J_0 = J_1 = JF; JF = 0: any J, c_0 is loaded in the round.
+constexpr int kBatchWarps2d = 2;
+// Batches take k_gridding_chunk2d below this mean chunk and above this many CTAs.
+// Measured, k_gridding_chunk2d against k_gridding_chunk_staged: 30 points per
+// chunk, 32 coils 76 us against 95; 108 points, 16 images 55 against 46; 105
+// points, 8 coils (1968 CTAs) 20 against 14.
+constexpr int64_t kBatchMaxMean = 64;
+constexpr int64_t kBatchMinCtas = 32 * 152;
+struct Tile2d {
+  int org0, org1;   // tile origin on the grid
+};
+__device__ __forceinline__ Tile2d tile_origin2d(const Geom& g, int bin) {
+  const int b0 = bin / g.nb[1];
+  return {b0 * g.T[0], (bin - b0 * g.nb[1]) * g.T[1]};
+}
+
+template <int JF>
+__host__ __device__ inline int strip2d(int J0, int J1) { return (JF > 0 ? JF : J0) * (32 / (JF > 0 ? JF : J1)); }
+
+// Runs body(cur, q, base, c1) for the warp's rounds of points: cur = the lane
+// has a point, q = its index in the chunk, base = the padded-tile cell of the
+// lane's column in the point's first row, c1 = c_1[l]; c_0[j] of the lane's
+// point is strip[j * PW + sub].
+template <int JF, class Body>
+__device__ __forceinline__ void for_points2d(const Chunk& ch, const Points& P, const Geom& g, const Tile2d T,
+                                             float2* strip, Body body) {
+  const int J0 = JF > 0 ? JF : g.J[0];
+  const int G = JF > 0 ? JF : g.J[1];
+  const int PW = 32 / G;
+  const int lane = threadIdx.x & 31;
+  const int sub = lane / G;
+  const int l = lane - sub * G;
+  const int step = (blockDim.x >> 5) * PW;
+  const int64_t M = P.M;
+  const float2* pc0 = P.coef + P.coef_off[0] + ch.start + (JF > 0 ? (int64_t)l * M : 0);
+  const float2* pc1 = P.coef + P.coef_off[1] + (int64_t)l * M + ch.start;
+  const int32_t* pk = P.kf + ch.start;
+  int qb = (threadIdx.x >> 5) * PW;
+  bool act = sub < PW && qb + sub < ch.count;
+  float2 n0 = make_float2(0.f, 0.f), n1 = n0;
+  int k0 = 0, k1 = 0;
+  if (act) {
+    const int q = qb + sub;
+    if (JF > 0) n0 = pc0[q];
+    n1 = pc1[q];
+    k0 = pk[q];
+    k1 = pk[M + q];
+  }
+  for (; qb < ch.count; qb += step) {   // warp-uniform
+    const bool cur = act;
+    const int q = qb + sub;
+    const float2 c1 = n1;
+    int base = 0;
+    __syncwarp();   // the strip's readers of the previous round are done
+    if (cur) {
+      if (JF > 0) {
+        strip[l * PW + sub] = n0;
+      } else {
+        for (int j = l; j < J0; j += G) strip[j * PW + sub] = pc0[(int64_t)j * M + q];
+      }
+      base = (k0 - T.org0) * g.P[1] + k1 - T.org1 + l;
+    }
+    const int qn = q + step;
+    act = sub < PW && qn < ch.count;
+    if (act) {
+      if (JF > 0) n0 = pc0[qn];
+      n1 = pc1[qn];
+      k0 = pk[qn];
+      k1 = pk[M + qn];
+    }
+    __syncwarp();
+    body(cur, q, base, c1);
+  }
+}
+
+// V^H (fixed-point accumulation as in k_gridding_chunk; the samples wait in
+// shared memory after the pass that finds the scale).  Shared memory: the two
+// accumulator planes, the samples, the strips.
+template <int JF>
+__global__ void __launch_bounds__(32 * kBatchWarps2d)
+k_gridding_chunk2d(const float2* __restrict__ y_b, float2* __restrict__ tiles_b, const Chunk* __restrict__ chunks,
+                   const Points P, const Geom g, int64_t ybs, int64_t tbs) {
+  extern __shared__ int acc[];
+  __shared__ float red[32];
+  const float2* __restrict__ y = y_b + (int64_t)blockIdx.y * ybs;
+  float2* __restrict__ tiles = tiles_b + (int64_t)blockIdx.y * tbs;
+  const int ncell = (int)g.padded_cells;
+  float2* s_y = reinterpret_cast<float2*>(acc + 2 * ncell);   // 8-byte aligned: 2 * ncell words
+  float2* strip = s_y + kChunkPoints[2] + (threadIdx.x >> 5) * strip2d<JF>(g.J[0], g.J[1]);
+  const Chunk ch = chunks[blockIdx.x];
+  const Tile2d T = tile_origin2d(g, ch.bin);
+  float mag = 0.f;
+  for (int q = threadIdx.x; q < ch.count; q += blockDim.x) {
+    const float2 v = __ldg(&y[P.perm[ch.start + q]]);
+    s_y[q] = v;
+    mag += fabsf(v.x) + fabsf(v.y);
+  }
+  for (int c = threadIdx.x; c < ncell; c += blockDim.x) reinterpret_cast<int2*>(acc)[c] = make_int2(0, 0);
+  // the sum also orders the zeroing and s_y before their use
+  const ChunkScale cs = chunk_scale<2>(block_sum_fixed(mag, red), P.cmax);
+  if (cs.finite) {   // CTA-uniform
+    const int J0 = JF > 0 ? JF : g.J[0];
+    const int PW = 32 / (JF > 0 ? JF : g.J[1]);
+    const int sub = (threadIdx.x & 31) / (JF > 0 ? JF : g.J[1]);
+    const int P1 = g.P[1];
+    for_points2d<JF>(ch, P, g, T, strip, [&](bool cur, int q, int base, float2 c1) {
+      if (!cur) return;
+      const float2 yl = cmulc(c1, cscale(s_y[q], cs.S));   // conj(c_last) * y * S
+#pragma unroll
+      for (int j0 = 0; j0 < (JF > 0 ? JF : kMaxJ); ++j0) {
+        if (JF == 0 && j0 >= J0) break;
+        const float2 w = cmulc(strip[j0 * PW + sub], yl);
+        int* cell = acc + base + j0 * P1;
+        atomicAdd(cell, __float2int_rn(w.x));
+        atomicAdd(cell + ncell, (j0 & 1) ? round_int(w.y) : __float2int_rn(w.y));   // see scatter_chunk3d
+      }
+    });
+  }
+  __syncthreads();
+  float2* out = tiles + (int64_t)ch.slot * g.padded_cells;
+  for (int c = threadIdx.x; c < ncell; c += blockDim.x) out[c] = fix_value<2>(acc, ncell, c, cs);
+}
+
+// 2D, batches: thread (r1, z0) of a tile sums the cells r0 = z0 .. z0 + 7 of its
+// column, as k_gridding_reduce3d below does, so a 16^2 tile takes one warp and a
+// CTA several tiles.  The same sums in the same order as reduce_tile with one
+// group.  A frame of 32 coils on a 512^2 grid (32 x 1024 tiles): 55 us with 64
+// threads and a neighbour mask per cell.
+constexpr int kRed2Rows = 8;
+constexpr int kRed2Threads = 256;
+
+__global__ void __launch_bounds__(kRed2Threads)
+k_gridding_reduce2d(const float2* __restrict__ tiles_b, const int32_t* __restrict__ bin_chunk,
+                    float2* __restrict__ grid_b, const Geom g, int64_t tbs, int64_t gbs, int nz) {
+  const float2* __restrict__ tiles = tiles_b + (int64_t)blockIdx.y * tbs;
+  float2* __restrict__ grid = grid_b + (int64_t)blockIdx.y * gbs;
+  const int T0 = g.T[0], T1 = g.T[1], P1 = g.P[1];
+  const int item = blockIdx.x * kRed2Threads + threadIdx.x;   // (tile, z, r1)
+  const int tz = item / T1, r1 = item - tz * T1;
+  const int bin = tz / nz, z0 = (tz - bin * nz) * kRed2Rows;
+  if (bin >= (int)g.nbins) return;   // no barriers below
+  const int b0 = bin / g.nb[1], b1 = bin - b0 * g.nb[1];
+  const int nzc = min(kRed2Rows, T0 - z0);
+  float2 acc[kRed2Rows];
+#pragma unroll
+  for (int k = 0; k < kRed2Rows; ++k) acc[k] = make_float2(0.f, 0.f);
+#pragma unroll 1
+  for (int e = 0; e < 4; ++e) {
+    const int e0 = e >> 1, e1 = e & 1;
+    const int n = e0 ? min(nzc, g.J[0] - 1 - z0) : nzc;   // the neighbour below reaches r0 < J - 1
+    if (n <= 0 || (e1 && r1 >= g.J[1] - 1)) continue;
+    const int s0 = e0 ? (b0 > 0 ? b0 : g.nb[0]) - 1 : b0;
+    const int s1 = e1 ? (b1 > 0 ? b1 : g.nb[1]) - 1 : b1;
+    const int src = s0 * g.nb[1] + s1;
+    const int q1 = __ldg(&bin_chunk[src + 1]);
+    int q = __ldg(&bin_chunk[src]);
+    const float2* ptr = tiles + (int64_t)q * g.padded_cells + (z0 + e0 * T0) * P1 + r1 + e1 * T1;
+    for (; q < q1; ++q, ptr += g.padded_cells) {
+      float2 v[kRed2Rows];
+#pragma unroll
+      for (int k = 0; k < kRed2Rows; ++k) v[k] = k < n ? __ldg(&ptr[k * P1]) : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < kRed2Rows; ++k)
+        if (k < n) acc[k] = cadd(acc[k], v[k]);
+    }
+  }
+  float2* out = grid + ((b0 * T0 + z0) * (int)g.Kstride[0] + b1 * T1 + r1);
+#pragma unroll
+  for (int k = 0; k < kRed2Rows; ++k)
+    if (k < nzc) out[k * (int)g.Kstride[0]] = acc[k];
+}
+
 // 3D: thread (r1, r2) of a tile sums kRed3Planes cells of its column, r0 = z0 ..
 // z0 + kRed3Planes - 1, so one address and one neighbour test serve the whole
 // column, its loads are all in flight together, and a warp of rows r1 >= J - 1
@@ -1300,7 +1531,7 @@ k_gridding_chunk_staged(const float2* __restrict__ y_b, float2* __restrict__ til
 constexpr int kRed3Planes = 8;
 constexpr int kRed3Threads = 256;
 
-__global__ void __launch_bounds__(kRed3Threads)
+__global__ void __launch_bounds__(kRed3Threads, 4)
 k_gridding_reduce3d(const float2* __restrict__ tiles_b, const int32_t* __restrict__ bin_chunk,
                     float2* __restrict__ grid_b, const Geom g, int64_t tbs, int64_t gbs, int nsl, int nz) {
   const float2* __restrict__ tiles = tiles_b + (int64_t)blockIdx.y * tbs;
@@ -1317,7 +1548,7 @@ k_gridding_reduce3d(const float2* __restrict__ tiles_b, const int32_t* __restric
   float2 acc[kRed3Planes];
 #pragma unroll
   for (int k = 0; k < kRed3Planes; ++k) acc[k] = make_float2(0.f, 0.f);
-#pragma unroll
+#pragma unroll 1
   for (int e = 0; e < 8; ++e) {
     const int e0 = e >> 2, e1 = (e >> 1) & 1, e2 = e & 1;
     const int n = e0 ? min(nzc, g.J[0] - 1 - z0) : nzc;   // the neighbour below reaches r0 < J - 1
@@ -1369,6 +1600,16 @@ cudaError_t launch_reduce(const nufft_plan_t* p, const float2* tiles, float2* gr
     k_gridding_reduce3d<<<dim3((unsigned)(g.nbins * nsl), (unsigned)nb), threads, 0, p->stream>>>(
         tiles, p->bin_chunk, grid, g, p->nchunks * g.padded_cells, p->Kprod, nsl, nz);
     return cudaGetLastError();
+  }
+  if constexpr (D == 2) {
+    if (nb > 1) {
+      const Geom& g = p->g;
+      const int nz = (g.T[0] + kRed2Rows - 1) / kRed2Rows;
+      const int64_t items = g.nbins * nz * g.T[1];
+      k_gridding_reduce2d<<<dim3((unsigned)((items + kRed2Threads - 1) / kRed2Threads), (unsigned)nb), kRed2Threads, 0,
+                            p->stream>>>(tiles, p->bin_chunk, grid, g, p->nchunks * g.padded_cells, p->Kprod, nz);
+      return cudaGetLastError();
+    }
   }
   int cells = 1;
   for (int a = 0; a < D; ++a) cells *= p->g.T[a];
@@ -1461,8 +1702,21 @@ cudaError_t interp_d(const nufft_plan_t* p, const float2* grid, float2* y, int n
   const int64_t warps = (P.M + per_warp - 1) / per_warp;
   const int64_t blocks = (warps * 32 + 255) / 256;
   if (blocks == 0) return cudaSuccess;
+  if constexpr (D == 2) {
+    const dim3 gb((unsigned)blocks, (unsigned)((nb + kBatchPer - 1) / kBatchPer));
+    auto go = [&](auto kern) {
+      kern<<<gb, 256, 0, p->stream>>>(grid, y, P, p->g, p->Kprod, p->M, nb);
+      return cudaGetLastError();
+    };
+    switch (p->g.J[0] == p->g.J[1] ? p->g.J[0] : 0) {
+      case 4: return go(k_interp_batch2d<4>);
+      case 5: return go(k_interp_batch2d<5>);
+      case 6: return go(k_interp_batch2d<6>);
+      case 7: return go(k_interp_batch2d<7>);
+    }
+  }
   const dim3 gd((unsigned)blocks, (unsigned)nb);
-  auto kern = all_j_equal(p->g, 6) ? k_interp<D, 6> : k_interp<D, 0>;
+  auto kern = D != 2 && all_j_equal(p->g, 6) ? k_interp<D, (D != 2 ? 6 : 0)> : k_interp<D, 0>;
   kern<<<gd, 256, 0, p->stream>>>(grid, y, P, p->g, p->Kprod, p->M);
   return cudaGetLastError();
 }
@@ -1494,6 +1748,27 @@ cudaError_t launch_chunks(const nufft_plan_t* p, const float2* y, float2* tiles,
   const dim3 gd((unsigned)p->nchunks, (unsigned)nb);
   const bool j6 = all_j_equal(p->g, 6);
   cudaError_t e;
+  if constexpr (D == 2 && !FUSED) {
+    // few points per chunk and CTAs enough: two warps per CTA
+    if (p->nchunks * nb >= kBatchMinCtas && p->M <= kBatchMaxMean * p->nchunks) {
+      auto go = [&](auto kern, int nstrip) {
+        const size_t smem = (size_t)p->g.padded_cells * Fix<2>::kWords * sizeof(int) +
+                            ((size_t)kChunkPoints[2] + (size_t)kBatchWarps2d * nstrip) * sizeof(float2);
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        kern<<<gd, 32 * kBatchWarps2d, smem, p->stream>>>(y, tiles, p->chunks, P, p->g, ybs, tbs);
+        return cudaGetLastError();
+      };
+      const int J0 = p->g.J[0], J1 = p->g.J[1];
+      switch (J0 == J1 ? J0 : 0) {
+        case 4: return go(k_gridding_chunk2d<4>, strip2d<4>(J0, J1));
+        case 5: return go(k_gridding_chunk2d<5>, strip2d<5>(J0, J1));
+        case 6: return go(k_gridding_chunk2d<6>, strip2d<6>(J0, J1));
+        case 7: return go(k_gridding_chunk2d<7>, strip2d<7>(J0, J1));
+        default: return go(k_gridding_chunk2d<0>, strip2d<0>(J0, J1));
+      }
+    }
+  }
   if constexpr (D == 2) {
     const int sj = p->g.J[0] + p->g.J[1];
     const size_t smem = (size_t)p->g.padded_cells * Fix<2>::kWords * sizeof(int) +
