@@ -461,6 +461,10 @@ __global__ void k_coef_max(const float2* coef, int64_t M, int d, int J0, int J1,
 // points of at most 2^20 + 1: no overflow), so W does not depend on the order
 // of the atomics.  Lane layout and bank order are the gridding's; one atomic
 // and no samples, so about a third of its time.
+// JF > 0: every J is JF, the axis-1 magnitudes sit in registers.  A weight w < 2^21
+// is rounded up by adding 2^23 towards +infinity: the low mantissa bits are the
+// integer, no conversion instruction.
+template <int JF>
 __global__ void __launch_bounds__(512)
 k_chunk_wmax(Chunk* chunks, const int32_t* kf, const float2* coef, int64_t off1, int64_t off2, int64_t M, const Geom g,
              const uint32_t* cmax) {
@@ -473,7 +477,7 @@ k_chunk_wmax(Chunk* chunks, const int32_t* kf, const float2* coef, int64_t off1,
   if (threadIdx.x == 0) top = 0;
   __syncthreads();
   const float cb = __uint_as_float(cmax[0]) * __uint_as_float(cmax[1]) * __uint_as_float(cmax[2]) * (1.f + 0x1p-20f);
-  const float sc = cb > 0.f ? 0x1p20f / cb : 0.f;
+  const float sc = cb > 0.f ? 0x1p20f / cb * (1.f - 0x1p-22f) : 0.f;   // w <= 2^20
   int org[kMaxDim];
   {
     int rem = ch.bin;
@@ -482,21 +486,30 @@ k_chunk_wmax(Chunk* chunks, const int32_t* kf, const float2* coef, int64_t off1,
       rem /= g.nb[a];
     }
   }
-  const int G = g.J[2], lane = threadIdx.x & 31, per_warp = 32 / G, sub = lane / G, l = lane - sub * G;
+  auto mag = [](float2 c) { return sqrtf(c.x * c.x + c.y * c.y); };
+  const int G = JF > 0 ? JF : g.J[2], J0 = JF > 0 ? JF : g.J[0], J1 = JF > 0 ? JF : g.J[1];
+  const int lane = threadIdx.x & 31, per_warp = 32 / G, sub = lane / G, l = lane - sub * G;
   if (sub < per_warp) {
     for (int q = (threadIdx.x >> 5) * per_warp + sub; q < ch.count; q += (blockDim.x >> 5) * per_warp) {
       const int64_t i = (int64_t)ch.start + q;
-      const float2 c2 = coef[off2 + (int64_t)l * M + i];
-      const float w2 = sqrtf(c2.x * c2.x + c2.y * c2.y) * sc;
+      const float w2 = mag(coef[off2 + (int64_t)l * M + i]) * sc;
       const int l0 = kf[i] - org[0], l1 = kf[M + i] - org[1], ll = kf[2 * M + i] - org[2] + l;
-      for (int j0 = 0; j0 < g.J[0]; ++j0) {
-        const float2 c0 = coef[(int64_t)j0 * M + i];
-        const float w0 = sqrtf(c0.x * c0.x + c0.y * c0.y) * w2;
-        for (int j1 = 0; j1 < g.J[1]; ++j1) {
-          const float2 c1 = coef[off1 + (int64_t)j1 * M + i];
-          const float w = sqrtf(c1.x * c1.x + c1.y * c1.y) * w0;
-          atomicAdd(&wacc[((l0 + j0) * g.P[1] + l1 + j1) * g.P[2] + ll],
-                    min((uint32_t)ceilf(w * (1.f + 0x1p-20f)), (1u << 20) + 1u));
+      float m0[JF > 0 ? JF : 1], m1[JF > 0 ? JF : 1];
+#pragma unroll
+      for (int j = 0; j < JF; ++j) {
+        m0[j] = mag(coef[(int64_t)j * M + i]);
+        m1[j] = mag(coef[off1 + (int64_t)j * M + i]);
+      }
+#pragma unroll
+      for (int j0 = 0; j0 < (JF > 0 ? JF : kMaxJ); ++j0) {
+        if (JF == 0 && j0 >= J0) break;
+        const float w0 = (JF > 0 ? m0[j0] : mag(coef[(int64_t)j0 * M + i])) * w2;
+        uint32_t* row = wacc + ((l0 + j0) * g.P[1] + l1) * g.P[2] + ll;
+#pragma unroll
+        for (int j1 = 0; j1 < (JF > 0 ? JF : kMaxJ); ++j1) {
+          if (JF == 0 && j1 >= J1) break;
+          const float w = __fmaf_ru(JF > 0 ? m1[j1] : mag(coef[off1 + (int64_t)j1 * M + i]), w0, 8388608.0f);
+          atomicAdd(row + j1 * g.P[2], __float_as_uint(w) & 0x7fffffu);
         }
       }
     }
@@ -507,7 +520,8 @@ k_chunk_wmax(Chunk* chunks, const int32_t* kf, const float2* coef, int64_t off1,
   m = __reduce_max_sync(0xffffffffu, m);
   if (lane == 0) atomicMax(&top, m);
   __syncthreads();
-  if (threadIdx.x == 0) chunks[blockIdx.x].wmax = __float_as_int(__uint2float_ru(top) * (0x1p-20f * cb) * (1.f + 0x1p-20f));
+  // undo the scaling; 1 + 2^-18 covers the roundings of the magnitudes and products
+  if (threadIdx.x == 0) chunks[blockIdx.x].wmax = __float_as_int(__uint2float_ru(top) * (0x1p-20f * cb) * (1.f + 0x1p-18f));
 }
 
 // Order each chunk's points for the gridding kernel.  Lane groups of J_last
@@ -822,8 +836,14 @@ int build_points(nufft_plan_t* p, const float* om) {
     NUFFT_CUDA_TRY(p, cudaGetLastError());
     if (d == 3 && nch > 0) {
       const size_t smem = (size_t)g.padded_cells * sizeof(uint32_t);
-      NUFFT_CUDA_TRY(p, cudaFuncSetAttribute(k_chunk_wmax, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      k_chunk_wmax<<<(unsigned)nch, 512, smem, st>>>(p->chunks, p->kf, p->coef, p->coef_off[1], p->coef_off[2], M, g,
+      const bool eq = g.J[0] == g.J[1] && g.J[1] == g.J[2];
+      auto kern = k_chunk_wmax<0>;
+      if (eq && g.J[0] == 4) kern = k_chunk_wmax<4>;
+      if (eq && g.J[0] == 5) kern = k_chunk_wmax<5>;
+      if (eq && g.J[0] == 6) kern = k_chunk_wmax<6>;
+      if (eq && g.J[0] == 7) kern = k_chunk_wmax<7>;
+      NUFFT_CUDA_TRY(p, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      kern<<<(unsigned)nch, 512, smem, st>>>(p->chunks, p->kf, p->coef, p->coef_off[1], p->coef_off[2], M, g,
                                                      p->cmax);
       NUFFT_CUDA_TRY(p, cudaGetLastError());
     }
