@@ -23,8 +23,10 @@
 // are; the hand-offs between stages go through two shared-memory buffers used
 // in turn (one buffer where there is one hand-off), one barrier per hand-off.
 // Twiddles are computed in registers.
-// Other line lengths (even, prime factors 2, 3 and 5) run a Stockham FFT of
-// radix-8, -4/-2, -3 and -5 stages through shared memory (k_fft_mixed).
+// Other line lengths (even, prime factors 2, 3 and 5) run stages of radices 2 to 16
+// (k_fft_mixed).
+#include <type_traits>
+
 #include "internal.cuh"
 
 namespace nufft {
@@ -63,9 +65,15 @@ struct FftArgs {
 // shuffle tree per warp, then the warps in order.  Every thread must call it;
 // every thread gets the sum.  red: 32 doubles of shared scratch.
 __device__ __forceinline__ double block_sum_dbl(double v, double* red) {
+  const int lane = threadIdx.x & 31;
+  const int n = min(32, (int)blockDim.x - (int)(threadIdx.x & ~31u));   // lanes of this warp
+  const unsigned mask = n == 32 ? 0xffffffffu : (1u << n) - 1u;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  for (int o = 16; o > 0; o >>= 1) {   // lane 0 ends with the sum of the lanes there are
+    const double u = __shfl_xor_sync(mask, v, o);
+    v += (lane ^ o) < n ? u : 0.0;
+  }
+  if (lane == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
   double t = 0.0;
   const int nw = (blockDim.x + 31) >> 5;
@@ -489,33 +497,61 @@ cudaError_t launch_L(const FftArgs& A, int nb, cudaStream_t st, int64_t* nblocks
 }
 
 // ---------------------------------------------------------------- other line lengths
-// Stockham FFT of a line of length L = 2^a 3^b 5^c through shared memory:
-// radix-8 stages, one radix-4 or radix-2 stage, then radix-3 and radix-5
-// stages.  Stage s of radix R and span Ns (the product of the earlier radices)
-// takes butterfly j (0 <= j < L/R) from elements j + r L/R, multiplies input
-// r by exp(-+ 2 pi i r k / (Ns R)), k = j mod Ns, transforms the R values and
-// writes output r to (j - k) R + k + r Ns.  The line sits in shared memory
-// (two buffers used in turn, one barrier per stage); loads and stores are
-// pruned and scaled as in k_fft_pass.
-constexpr int kMaxStages = 16;
+// Lines of length L = 2^a 3^b 5^c: a Stockham FFT.  Stage s of radix R and span Ns
+// (the product of the earlier radices) takes butterfly j (0 <= j < L/R) from
+// elements j + r L/R, multiplies input r by exp(-+ 2 pi i r k / (Ns R)), k = j mod
+// Ns, transforms the R values and writes output r to (j - k) R + k + r Ns.  The
+// first stage reads global memory and the last one writes it (its outputs are
+// j + r Ns), both pruned and scaled as in k_fft_pass; the hand-offs between go
+// through two shared-memory buffers used in turn, one barrier each.
+// Radices 8 to 2 only: with 9, 10, 12, 15 and 16 too (two or three stages for
+// every L) the passes were slower at every size, from a 54^2 grid (136 us for an
+// 8-coil CG against 143) to 16 transforms of 384^2 (pair 151 us against 164):
+// more registers, fewer threads per line and more code.
+constexpr int kMaxStages = 5;
 struct MixedRadix {
   int L;
   int nst;
   int radix[kMaxStages];
+  int ns[kMaxStages];          // span of the stage
+  uint32_t magic[kMaxStages];  // ceil(2^32 / ns): j / ns = umulhi(j, magic) for 1 < ns, j < 2^10
+  float step[kMaxStages];      // 2 / (ns radix), the twiddles' angle per k in units of pi,
+  float step_lo[kMaxStages];   // and what its rounding left
 };
 
+// Fewest stages, then the smallest largest radix; radices in descending order
+// (the first stage has no twiddles).
+void mixed_search(const int* set, int nset, int rest, int depth, int limit, int* cur, MixedRadix* best) {
+  if (rest == 1) {
+    if (depth > 0 && (best->nst < 0 || depth < best->nst || (depth == best->nst && cur[0] < best->radix[0]))) {
+      best->nst = depth;
+      for (int i = 0; i < depth; ++i) best->radix[i] = cur[i];
+    }
+    return;
+  }
+  if (depth == kMaxStages) return;
+  for (int i = 0; i < nset; ++i) {
+    if (set[i] > limit || rest % set[i] != 0) continue;
+    cur[depth] = set[i];
+    mixed_search(set, nset, rest / set[i], depth + 1, set[i], cur, best);
+  }
+}
+
 MixedRadix mixed_radix(int L) {
+  static const int kRadix[] = {8, 6, 5, 4, 3, 2};
   MixedRadix m;
   memset(&m, 0, sizeof(m));
   m.L = L;
-  int a = 0, v = L;
-  while (v % 2 == 0) { v /= 2; ++a; }
-  for (int i = 0; i < a / 3; ++i) m.radix[m.nst++] = 8;
-  if (a % 3 == 2) m.radix[m.nst++] = 4;
-  if (a % 3 == 1) m.radix[m.nst++] = 2;
-  while (v % 3 == 0) { v /= 3; m.radix[m.nst++] = 3; }
-  while (v % 5 == 0) { v /= 5; m.radix[m.nst++] = 5; }
-  if (v != 1) m.nst = -1;   // not a supported length
+  m.nst = -1;
+  int cur[kMaxStages];
+  mixed_search(kRadix, 6, L, 0, 8, cur, &m);
+  for (int s = 0, ns = 1; s < m.nst; ns *= m.radix[s++]) {
+    m.ns[s] = ns;
+    m.magic[s] = (uint32_t)((0x100000000ull + ns - 1) / ns);
+    const double step = 2.0 / ((double)ns * m.radix[s]);
+    m.step[s] = (float)step;
+    m.step_lo[s] = (float)(step - (double)m.step[s]);
+  }
   return m;
 }
 
@@ -552,189 +588,293 @@ __device__ __forceinline__ void dft5(float2* v) {
   v[3] = csub(a2, b2);
 }
 
-template <bool STRIDED>
-struct MixedMap {
-  int w, L;   // lines per CTA, line length
-  __device__ __forceinline__ int at(int b, int p) const { return STRIDED ? p * (w + 1) + b : b * (L + 1) + p; }
-  __host__ __device__ static size_t words(int w, int L) { return (size_t)(STRIDED ? L * (w + 1) : w * (L + 1)); }
-};
+template <int R, bool INV>
+__device__ __forceinline__ void dft_any(float2* v);
 
-template <int R, bool INV, bool STRIDED>
-__device__ __forceinline__ void mixed_stage(const float2* __restrict__ src, float2* __restrict__ dst,
-                                            const MixedMap<STRIDED> SI, int b, int t, int TPL, int Ns) {
-  const int L = SI.L;
-  const int nbf = L / R;
-  const float inv = 2.0f / (float)(Ns * R);
-  for (int j = t; j < nbf; j += TPL) {
-    const int k = j % Ns;
-    float2 v[R];
+// DFT of N = N1 N2 points, N1 and N2 coprime, without twiddles (Good and Thomas):
+// input (N2 n1 + N1 n2) mod N, output (N2 u1 k1 + N1 u2 k2) mod N with
+// u1 = N2^-1 mod N1, u2 = N1^-1 mod N2.
+constexpr int inv_mod(int a, int m) {
+  for (int x = 1; x < m; ++x)
+    if (a * x % m == 1) return x;
+  return 0;
+}
+template <int N1, int N2, bool INV>
+__device__ __forceinline__ void dft_coprime(float2* v) {
+  constexpr int N = N1 * N2, u1 = inv_mod(N2 % N1, N1) * N2, u2 = inv_mod(N1 % N2, N2) * N1;
+  float2 a[N1][N2];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = src[SI.at(b, j + r * nbf)];
-    if (Ns > 1) {   // input r times w1^r, w1 = exp(-+ 2 pi i k / (Ns R)), computed (no table loads)
-      float sn, cs;
-      sincospif((float)k * inv, &sn, &cs);
-      const float2 w1 = make_float2(cs, INV ? sn : -sn);
-      float2 w = w1;
+  for (int i = 0; i < N1; ++i) {
 #pragma unroll
-      for (int r = 1; r < R; ++r) {
-        v[r] = cmul(v[r], w);
-        if (r + 1 < R) w = cmul(w, w1);
-      }
-    }
-    if (R == 3) dft3<INV>(v);
-    else if (R == 5) dft5<INV>(v);
-    else dft<R, INV>(v);
-    const int base = (j - k) * R + k;
+    for (int j = 0; j < N2; ++j) a[i][j] = v[(N2 * i + N1 * j) % N];
+    dft_any<N2, INV>(a[i]);
+  }
 #pragma unroll
-    for (int r = 0; r < R; ++r) dst[SI.at(b, base + r * Ns)] = v[r];
+  for (int j = 0; j < N2; ++j) {
+    float2 c[N1];
+#pragma unroll
+    for (int i = 0; i < N1; ++i) c[i] = a[i][j];
+    dft_any<N1, INV>(c);
+#pragma unroll
+    for (int i = 0; i < N1; ++i) v[(u1 * i + u2 * j) % N] = c[i];
   }
 }
 
-template <bool STRIDED, bool INV>
-__global__ void __launch_bounds__(256)
-k_fft_mixed(const FftArgs A, const int W, const __grid_constant__ MixedRadix mr) {
+template <int R, bool INV>
+__device__ __forceinline__ void dft_any(float2* v) {
+  if constexpr (R == 2) dft2<INV>(v);
+  else if constexpr (R == 3) dft3<INV>(v);
+  else if constexpr (R == 5) dft5<INV>(v);
+  else if constexpr (R == 6) dft_coprime<2, 3, INV>(v);
+  else dft<R, INV>(v);
+}
+
+// exp(-+ i pi k (step + step_lo)): sincospif of the rounded angle, corrected to
+// first order for what the rounding left.
+template <bool INV>
+__device__ __forceinline__ float2 mixed_root(int k, float step, float step_lo) {
+  const float kf = (float)k, a = kf * step;
+  const float d = 3.14159265358979f * (fmaf(kf, step, -a) + kf * step_lo);
+  float sn, cs;
+  sincospif(a, &sn, &cs);
+  const float c1 = fmaf(-sn, d, cs), s1 = fmaf(cs, d, sn);
+  return make_float2(c1, INV ? s1 : -s1);
+}
+
+// Input r of a butterfly times w1^r, w1 = exp(-+ i pi k step): w1, for R >= 5 also
+// w1^2 (a power multiplies the root's error, and a second root halves the powers),
+// and products of depth at most three.
+template <int R, bool INV>
+__device__ __forceinline__ void mixed_twiddles(float2* v, int k, float step, float step_lo) {
+  float2 w[8];
+  w[1] = mixed_root<INV>(k, step, step_lo);
+  if (R >= 5) w[2] = mixed_root<INV>(2 * k, step, step_lo);
+#pragma unroll
+  for (int r = 1; r < R; ++r) {
+    if (r > 2 || (r == 2 && R < 5)) w[r] = cmul(w[r / 2], w[r - r / 2]);
+    v[r] = cmul(v[r], w[r]);
+  }
+}
+
+// Shared-memory position of element p of line b: strided axis, rows of W columns
+// (a skewed row for fewer than 16, so that the threads of a half-warp in
+// neighbouring rows differ mod 16); contiguous axis, one pad word per 8.
+template <bool STRIDED>
+struct MixedMap {
+  int wlog, pitch;
+  __device__ __forceinline__ MixedMap(int wl, int L) : wlog(wl), pitch(L + (L >> 3) + 1) {}
+  __device__ __forceinline__ int at(int b, int p) const {
+    return STRIDED ? ((wlog < 4 ? p + (p >> 3) : p) << wlog) + b : b * pitch + p + (p >> 3);
+  }
+  __host__ __device__ static size_t words(int wlog, int L) { return (size_t)(L + (L >> 3) + 1) << wlog; }
+};
+
+// f(integral_constant<int, R>) for a runtime radix R.
+template <class F>
+__device__ __forceinline__ void for_radix(int R, F f) {
+  switch (R) {
+    case 2: f(std::integral_constant<int, 2>{}); break;
+    case 3: f(std::integral_constant<int, 3>{}); break;
+    case 4: f(std::integral_constant<int, 4>{}); break;
+    case 5: f(std::integral_constant<int, 5>{}); break;
+    case 6: f(std::integral_constant<int, 6>{}); break;
+    default: f(std::integral_constant<int, 8>{}); break;
+  }
+}
+
+// grid: as k_fft_pass.  blockDim = TPL << wlog, TPL threads per line.
+template <bool STRIDED, bool INV, bool HOOK>
+__global__ void __launch_bounds__(512)
+k_fft_mixed(const FftArgs A, const int wlog, const __grid_constant__ MixedRadix mr) {
   const int L = mr.L;
-  const int TPL = blockDim.x / W;
-  const MixedMap<STRIDED> SI{W, L};
+  const int TPL = blockDim.x >> wlog;
+  const MixedMap<STRIDED> SI(wlog, L);
   extern __shared__ float2 sm[];
-  const int bufw = (int)MixedMap<STRIDED>::words(W, L);
 
   const int tid = threadIdx.x;
-  int b, t;
-  int64_t o, in;
+  int b, t, o, in;
   if (STRIDED) {
-    b = tid % W;
-    t = tid / W;
-    const int64_t nib = A.inner / W;
-    o = blockIdx.x / nib;
-    in = (blockIdx.x % nib) * W + b;
+    b = tid & ((1 << wlog) - 1);
+    t = tid >> wlog;
+    o = blockIdx.y;
+    in = (blockIdx.x << wlog) + b;
   } else {
     b = tid / TPL;
-    t = tid % TPL;
-    o = (int64_t)blockIdx.x * W + b;
+    t = tid - b * TPL;
+    o = (blockIdx.x << wlog) + b;
     in = 0;
   }
-  const bool live = o < A.nouter;
-  const float2* __restrict__ src = A.src + (int64_t)blockIdx.y * A.src_bstride;
-  float2* __restrict__ dst = A.dst + (int64_t)blockIdx.y * A.dst_bstride;
+  const bool live = o < (int)A.nouter;
+  const float2* __restrict__ src = A.src + (int64_t)blockIdx.z * A.src_bstride;
+  float2* __restrict__ dst = A.dst + (int64_t)blockIdx.z * A.dst_bstride;
 
-  int64_t goff = 0;
+  int goff = in;
   float slead = 1.0f;
   if (live) {
-    int64_t rem = o;
+    int rem = o;
     for (int i = A.a - 1; i >= 0; --i) {
-      const int n = (int)(rem % A.lead_N[i]);
-      rem /= A.lead_N[i];
+      int n = rem;
+      if (i > 0) {
+        rem = n / A.lead_N[i];
+        n -= rem * A.lead_N[i];
+      }
       const int gi = wrapk(n - A.lead_N[i] / 2 + A.lead_K[i], A.lead_K[i]);
-      goff += (int64_t)gi * A.lead_stride[i];
+      goff += gi * (int)A.lead_stride[i];
       if (A.scale && (A.src_image || A.dst_image)) slead *= A.s_lead[i][n];
     }
   }
   const int half = A.Na >> 1;
-  const int64_t stride = A.inner;
-  __shared__ double red[32];
-  const bool pro = !INV && A.src_image && A.pro_p;
-  const float beta = pro ? cg_prologue_beta(A, red) : 0.f;
+  const int stride = STRIDED ? (int)A.inner : 1;
+  const bool pro = HOOK && !INV && A.src_image && A.pro_p;
+  float beta = 0.f;
+  if constexpr (HOOK && !INV) {
+    __shared__ double red[32];
+    if (pro) beta = cg_prologue_beta(A, red);
+  }
   const uint64_t pol = l2_evict_first_policy();   // a pass reads each input element once
 
-  for (int p = t; p < L; p += TPL) {
-    float2 v = make_float2(0.f, 0.f);
-    if (live) {
-      if (!INV) {
-        if ((p < half) || (p >= L - half)) {
-          if (A.src_image) {
-            const int n = p < half ? p + half : p - L + half;
-            v = cscale(load_image(A, src, o * A.Na + n, pro, beta), (A.scale ? A.s_axis[n] : 1.0f) * slead);
-          } else {
-            v = ld_last_use(&src[goff + (int64_t)p * stride + in], pol);
+  // ---- first stage: global memory (pruned on the forward side) to buffer 0
+  auto first = [&](auto rc) {
+    constexpr int R = decltype(rc)::value;
+    const int nbf = L / R;
+    for (int j = t; j < nbf; j += TPL) {
+      float2 v[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int p = j + r * nbf;
+        v[r] = make_float2(0.f, 0.f);
+        if (live) {
+          if (INV) {
+            v[r] = ld_last_use(&src[goff + p * stride], pol);
+          } else if ((p < half) || (p >= L - half)) {
+            if (A.src_image) {
+              const int n = p < half ? p + half : p - L + half;
+              v[r] = cscale(load_image(A, src, o * A.Na + n, pro, beta), (A.scale ? A.s_axis[n] : 1.0f) * slead);
+            } else {
+              v[r] = ld_last_use(&src[goff + p * stride], pol);
+            }
           }
         }
-      } else {
-        v = ld_last_use(&src[goff + (int64_t)p * stride + in], pol);
       }
+      dft_any<R, INV>(v);
+#pragma unroll
+      for (int r = 0; r < R; ++r) sm[SI.at(b, j * R + r)] = v[r];
     }
-    sm[SI.at(b, p)] = v;
-  }
+  };
+  for_radix(mr.radix[0], first);
   __syncthreads();
 
-  int cur = 0, Ns = 1;
-  for (int s = 0; s < mr.nst; ++s) {
-    const int R = mr.radix[s];
-    const float2* in_buf = sm + cur * bufw;
-    float2* out_buf = sm + (cur ^ 1) * bufw;
-    switch (R) {
-      case 2: mixed_stage<2, INV>(in_buf, out_buf, SI, b, t, TPL, Ns); break;
-      case 3: mixed_stage<3, INV>(in_buf, out_buf, SI, b, t, TPL, Ns); break;
-      case 4: mixed_stage<4, INV>(in_buf, out_buf, SI, b, t, TPL, Ns); break;
-      case 5: mixed_stage<5, INV>(in_buf, out_buf, SI, b, t, TPL, Ns); break;
-      default: mixed_stage<8, INV>(in_buf, out_buf, SI, b, t, TPL, Ns); break;
-    }
+  // ---- middle stages, from one buffer to the other
+  float2* cur = sm;
+  float2* nxt = sm + MixedMap<STRIDED>::words(wlog, L);
+  for (int s = 1; s + 1 < mr.nst; ++s) {
+    const int Ns = mr.ns[s];
+    const uint32_t mg = mr.magic[s];
+    for_radix(mr.radix[s], [&](auto rc) {
+      constexpr int R = decltype(rc)::value;
+      const int nbf = L / R;
+      for (int j = t; j < nbf; j += TPL) {
+        const int k = j - (int)__umulhi((uint32_t)j, mg) * Ns;
+        float2 v[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = cur[SI.at(b, j + r * nbf)];
+        mixed_twiddles<R, INV>(v, k, mr.step[s], mr.step_lo[s]);
+        dft_any<R, INV>(v);
+        const int base = (j - k) * R + k;
+#pragma unroll
+        for (int r = 0; r < R; ++r) nxt[SI.at(b, base + r * Ns)] = v[r];
+      }
+    });
     __syncthreads();
-    cur ^= 1;
-    Ns *= R;
+    float2* const tmp = cur;
+    cur = nxt;
+    nxt = tmp;
   }
 
-  const float2* res = sm + cur * bufw;
-  const bool epi = INV && A.dst_image && A.epi_part;
+  // ---- last stage: to global memory (pruned on the inverse side); Ns = L / R, so
+  // k = j and output r is element j + r Ns
+  const bool epi = HOOK && INV && A.dst_image && A.epi_part;
   double dot = 0.0;
-  if (live) {
-    for (int p = t; p < L; p += TPL) {
-      const float2 v = res[SI.at(b, p)];
-      if (!INV) {
-        dst[goff + (int64_t)p * stride + in] = v;
-      } else {
-        if (!((p < half) || (p >= L - half))) continue;
-        if (A.dst_image) {
-          const int n = p < half ? p + half : p - L + half;
-          const float2 out = cscale(v, (A.scale ? A.s_axis[n] : 1.0f) * slead);
-          dst[o * A.Na + n] = out;
-          if (epi) {
-            const float2 a = A.epi_a[o * A.Na + n];
-            dot += (double)a.x * (double)out.x + (double)a.y * (double)out.y;
+  auto last = [&](auto rc) {
+    constexpr int R = decltype(rc)::value;
+    const int nbf = L / R;
+    for (int j = t; j < nbf; j += TPL) {
+      float2 v[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[r] = cur[SI.at(b, j + r * nbf)];
+      mixed_twiddles<R, INV>(v, j, mr.step[mr.nst - 1], mr.step_lo[mr.nst - 1]);
+      dft_any<R, INV>(v);
+      if (!live) continue;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int p = j + r * nbf;
+        if (!INV) {
+          dst[goff + p * stride] = v[r];
+        } else if ((p < half) || (p >= L - half)) {
+          if (A.dst_image) {
+            const int n = p < half ? p + half : p - L + half;
+            const float2 out = cscale(v[r], (A.scale ? A.s_axis[n] : 1.0f) * slead);
+            dst[o * A.Na + n] = out;
+            if (epi) {
+              const float2 a = A.epi_a[o * A.Na + n];
+              dot += (double)a.x * (double)out.x + (double)a.y * (double)out.y;
+            }
+          } else {
+            dst[goff + p * stride] = v[r];
           }
-        } else {
-          dst[goff + (int64_t)p * stride + in] = v;
         }
       }
     }
-  }
-  if (epi) {
-    const double tsum = block_sum_dbl(dot, red);
-    if (threadIdx.x == 0) A.epi_part[blockIdx.x] = tsum;
+  };
+  for_radix(mr.radix[mr.nst - 1], last);
+  if constexpr (HOOK && INV) {
+    __shared__ double red[32];
+    if (epi) {
+      const double tsum = block_sum_dbl(dot, red);
+      if (threadIdx.x == 0) A.epi_part[blockIdx.x] = tsum;
+    }
   }
 }
 
-// 256 threads per CTA: W lines of 256 / W threads (strided axes: W adjacent
-// columns, W | inner), W lowered while the launch would give fewer than two
-// CTAs per SM.
+// One thread per butterfly of the smallest radix (at most 256 per line), W lines
+// per CTA: up to 16 columns on a strided axis (W | inner), as many lines as give
+// 256 threads on the contiguous one; at most 512 threads, and W lowered while the
+// launch would give fewer than two CTAs per SM.
 template <bool STRIDED, bool INV>
 cudaError_t launch_mixed(int L, const FftArgs& A, int nb, cudaStream_t st, int64_t* nblocks, bool query) {
   const MixedRadix mr = mixed_radix(L);
-  if (mr.nst < 0) return cudaErrorInvalidValue;
-  int W;
+  if (mr.nst < 2) return cudaErrorInvalidValue;
+  const int tpl = std::min(256, L / mr.radix[mr.nst - 1]);
+  auto smem = [&](int wlog) {
+    return (size_t)std::min(2, mr.nst - 1) * MixedMap<STRIDED>::words(wlog, L) * sizeof(float2);
+  };
+  int wlog = 0;
   int64_t blocks;
   if (STRIDED) {
-    W = 8;
-    while (W > 1 && (A.inner % W != 0 || A.nouter * (A.inner / W) * nb < kTargetBlocks ||
-                     2 * MixedMap<STRIDED>::words(W, L) * sizeof(float2) > 160 * 1024))
-      W >>= 1;
-    blocks = A.nouter * (A.inner / W);
+    wlog = 4;
+    while (wlog > 0 && (A.inner % (1 << wlog) != 0 || A.nouter * (A.inner >> wlog) * nb < kTargetBlocks ||
+                        smem(wlog) > 100 * 1024 || (tpl << wlog) > 512))
+      --wlog;
+    blocks = A.nouter * (A.inner >> wlog);
   } else {
-    const int tpl = L >= 512 ? 128 : (L >= 128 ? 64 : 32);
-    W = 256 / tpl;
-    while (W > 1 && (A.nouter + W - 1) / W * nb < kTargetBlocks) W >>= 1;
-    blocks = (A.nouter + W - 1) / W;
+    while ((tpl << (wlog + 1)) <= 256) ++wlog;
+    while (wlog > 0 && ((A.nouter + (1 << wlog) - 1) >> wlog) * nb < kTargetBlocks) --wlog;
+    blocks = (A.nouter + (1 << wlog) - 1) >> wlog;
   }
   if (nblocks) *nblocks = blocks;
   if (query) return cudaSuccess;
-  const int threads = STRIDED ? 256 : W * (L >= 512 ? 128 : (L >= 128 ? 64 : 32));
-  const size_t smem = 2 * MixedMap<STRIDED>::words(W, L) * sizeof(float2);
-  cudaError_t e = cudaFuncSetAttribute(k_fft_mixed<STRIDED, INV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return e;
-  if (blocks == 0) return cudaSuccess;
-  k_fft_mixed<STRIDED, INV><<<dim3((unsigned)blocks, (unsigned)nb), threads, smem, st>>>(A, W, mr);
-  return cudaGetLastError();
+  auto go = [&](auto kern) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(wlog));
+    if (e != cudaSuccess || blocks == 0) return e;
+    const dim3 gd = STRIDED ? dim3((unsigned)(A.inner >> wlog), (unsigned)A.nouter, (unsigned)nb)
+                            : dim3((unsigned)blocks, 1, (unsigned)nb);
+    kern<<<gd, tpl << wlog, smem(wlog), st>>>(A, wlog, mr);
+    return cudaGetLastError();
+  };
+  if constexpr (!STRIDED) {
+    if (A.pro_p || A.epi_part) return go(k_fft_mixed<STRIDED, INV, true>);
+  }
+  return go(k_fft_mixed<STRIDED, INV, false>);
 }
 
 template <bool STRIDED, bool INV>

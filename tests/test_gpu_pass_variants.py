@@ -63,6 +63,33 @@ def test_fft_passes(nf, Kd, Nd):
         assert rel(plan.ifft_crop_rescale(dev(z)).cpu().numpy(), oracle.crop_rescale(p, oracle.fft_adjoint(z))) < TOL_FFT
 
 
+# lines that are not powers of two: every radix (3 to 16) as the first, the middle
+# and the last stage, on a contiguous and on a strided axis
+@pytest.mark.parametrize("L", [18, 20, 24, 30, 50, 54, 72, 108, 144, 150, 162, 192, 240, 250, 324, 360, 384, 400, 500,
+                               750, 768, 864, 960, 972, 1000])
+@pytest.mark.parametrize("other,strided", [(16, True), (80, True), (36, False)])
+def test_mixed_radix_lines(nf, L, other, strided):
+    Kd = (L, other) if strided else (other, L)
+    Nd = tuple(2 * max(1, K // 3) for K in Kd)
+    om = W.uniform_random_om(5, 2, seed=4)
+    p = oracle.make_plan(om, Nd, Kd, (4, 4))
+    x, z = cn(Nd, 8), cn(Kd, 9)
+    with nf.NufftPlan(dev(om), Nd, Kd, (4, 4)) as plan:
+        assert rel(plan.scale_pad_fft(dev(x)).cpu().numpy(), oracle.fft_forward(oracle.scale_pad(p, x))) < TOL_FFT
+        assert rel(plan.ifft_crop_rescale(dev(z)).cpu().numpy(), oracle.crop_rescale(p, oracle.fft_adjoint(z))) < TOL_FFT
+
+
+# the CG step's sums in the image-side passes, with CTAs of full and of part warps
+@pytest.mark.parametrize("Nd,Kd", [((12, 14), (20, 18)), ((24, 30), (36, 60)), ((40, 36), (64, 50)), ((50, 64), (100, 128))])
+def test_cg_hooks_in_the_passes(nf, Nd, Kd):
+    om = W.uniform_random_om(4 * Nd[0] * Nd[1], 2, seed=6)
+    p = oracle.make_plan(om, Nd, Kd, (6, 6))
+    y = cn(om.shape[0], 10)
+    with nf.NufftPlan(dev(om), Nd, Kd, (6, 6)) as plan:
+        got = plan.solve_cg(dev(y), maxiter=3).cpu().numpy()
+    assert rel(got, oracle.cg(p, y, np.zeros(Nd), 3)) < 10 * TOL_OP
+
+
 @pytest.mark.parametrize("J", [4, 5, 6, 7])
 @pytest.mark.parametrize("Kd,M", [((32, 32, 32), 1), ((32, 32, 32), 6001), ((20, 24, 36), 1279), ((16, 18, 50), 81)])
 def test_3d_interpolation_and_gridding(nf, J, Kd, M):
