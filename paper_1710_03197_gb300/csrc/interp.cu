@@ -475,84 +475,132 @@ k_interp_chunk3d(const float2* __restrict__ grid_b, float2* __restrict__ y_b, co
   }
 }
 
-// 2D: the chunk's point data are staged too (one thread per point: first
-// neighbours, the J0 + J1 coefficients and the permutation), so the CTA waits
-// for one round of global loads instead of one per pass of its warps over the
-// chunk; the gathers then read only shared memory.  Shared memory: the two
-// planes of the padded tile, c0[J0][cap], c1[cap][J1] (as in the gridding's
-// staged kernel), k[2][cap], perm[cap].
-template <int JF>
-__global__ void __launch_bounds__(256, 4)
-k_interp_chunk2d(const float2* __restrict__ grid_b, float2* __restrict__ y_b, const Chunk* __restrict__ chunks,
-                 const Points P, const Geom g, int64_t gbs, int64_t ybs) {
-  constexpr int cap = kChunkPoints[2];
-  static_assert(cap == 256, "one thread per staged point");
-  extern __shared__ float tile[];
-  const float2* __restrict__ grid = grid_b + (int64_t)blockIdx.y * gbs;
-  float2* __restrict__ y = y_b + (int64_t)blockIdx.y * ybs;
-  const int ncell = (int)g.padded_cells;
-  const int P1 = g.P[1];
-  const int J0 = JF > 0 ? JF : g.J[0];
-  const int J1 = JF > 0 ? JF : g.J[1];
-  float* gre = tile;
-  float* gim = tile + ncell;
-  float2* s_c = reinterpret_cast<float2*>(tile + 2 * ncell);   // 8-byte aligned: 2 * ncell floats
-  int* s_k = reinterpret_cast<int*>(s_c + (J0 + J1) * cap);
-  int* s_p = s_k + 2 * cap;
-  const Chunk ch = chunks[blockIdx.x];
-  const int org0 = ((ch.bin / g.nb[1]) % g.nb[0]) * g.T[0];
-  const int org1 = (ch.bin % g.nb[1]) * g.T[1];
-  for (int c = threadIdx.x; c < ncell; c += blockDim.x) {
-    const int r1 = c % P1, r0 = c / P1;
-    const float2 v = __ldg(&grid[(int64_t)wrapk(org0 + r0, g.K[0]) * g.Kstride[0] + wrapk(org1 + r1, g.K[1])]);
-    gre[c] = v.x;
-    gim[c] = v.y;
-  }
-  const int qs = threadIdx.x;
-  if (qs < ch.count) {
-    const int64_t i = (int64_t)ch.start + qs;
-    s_p[qs] = P.perm[i];
-    s_k[qs] = P.kf[i] - org0;
-    s_k[cap + qs] = P.kf[P.M + i] - org1;
-#pragma unroll
-    for (int r = 0; r < (JF > 0 ? JF : kMaxJ); ++r) {
-      if (JF == 0 && r >= J0) break;
-      s_c[r * cap + qs] = P.coef[P.coef_off[0] + (int64_t)r * P.M + i];
-    }
-#pragma unroll
-    for (int r = 0; r < (JF > 0 ? JF : kMaxJ); ++r) {
-      if (JF == 0 && r >= J1) break;
-      s_c[J0 * cap + qs * J1 + r] = P.coef[P.coef_off[1] + (int64_t)r * P.M + i];
-    }
-  }
-  __syncthreads();
+// ---------------------------------------------------------------- 2D chunks, staged
+// Single 2D transforms: the chunk's point data are staged in shared memory too,
+// one thread per point (first neighbours, the J0 + J1 coefficients, permutation
+// or sample), so a CTA waits for one round of global loads instead of one per
+// pass of its warps over the chunk.  Layout: c0[J0][cap] (row by row: the lanes
+// of a point read one value), c1[cap][J1 | 1] (point by point: the lanes of a
+// point read consecutive words; the odd pitch keeps the staging threads' stores
+// on distinct banks, 2- to 4-way conflicts otherwise), k[2][cap] (first neighbours
+// relative to the tile origin).
+// JF > 0: J0 = J1 = JF; TF > 0: 16^2 tiles, so that the rows of a point's
+// neighbours are immediate offsets.
+struct Tile2d {
+  int org0, org1;   // tile origin on the grid
+};
+__device__ __forceinline__ Tile2d tile_origin2d(const Geom& g, int bin) {
+  const int b0 = bin / g.nb[1];
+  return {b0 * g.T[0], (bin - b0 * g.nb[1]) * g.T[1]};
+}
 
-  const int G = J1;
+struct Staged2d {
+  float2* c0;
+  float2* c1;
+  int* k;
+  int pitch1;
+  // float2 of shared memory per chunk for the coefficients
+  static size_t coefs(int J0, int J1) { return (size_t)kChunkPoints[2] * (J0 + (J1 | 1)); }
+};
+
+template <int JF>
+__device__ __forceinline__ void stage_points2d(const Staged2d& S, const Points& P, const Geom& g, const Chunk& ch,
+                                               const Tile2d T) {
+  constexpr int cap = kChunkPoints[2];
+  const int J0 = JF > 0 ? JF : g.J[0], J1 = JF > 0 ? JF : g.J[1];
+  const int q = threadIdx.x;
+  if (q >= ch.count) return;
+  const int i = ch.start + q;
+  S.k[q] = P.kf[i] - T.org0;
+  S.k[cap + q] = P.kf[P.M + i] - T.org1;
+  const float2* c0 = P.coef + P.coef_off[0] + i;
+  const float2* c1 = P.coef + P.coef_off[1] + i;
+#pragma unroll
+  for (int r = 0; r < (JF > 0 ? JF : kMaxJ); ++r) {
+    if (JF == 0 && r >= J0) break;
+    S.c0[r * cap + q] = c0[r * P.M];
+  }
+#pragma unroll
+  for (int r = 0; r < (JF > 0 ? JF : kMaxJ); ++r) {
+    if (JF == 0 && r >= J1) break;
+    S.c1[q * S.pitch1 + r] = c1[r * P.M];
+  }
+}
+
+// The chunk's padded tile of the grid into planes of real and imaginary parts,
+// one row per warp step.
+template <int PF>
+__device__ __forceinline__ void stage_tile2d(const float2* __restrict__ grid, const Geom& g, const Tile2d T, float* gre,
+                                             float* gim) {
+  const int P0 = PF > 0 ? PF : g.P[0], P1 = PF > 0 ? PF : g.P[1];
   const int lane = threadIdx.x & 31;
-  const int per_warp = 32 / G;
+  constexpr int kWarps = kChunkPoints[2] / 32;
+#pragma unroll(PF > 0 ? (PF + 7) / 8 : 1)
+  for (int r0 = threadIdx.x >> 5; r0 < P0; r0 += kWarps) {
+    const float2* src = grid + wrapk(T.org0 + r0, g.K[0]) * (int)g.Kstride[0];
+    for (int r1 = lane; r1 < P1; r1 += 32) {
+      const float2 v = __ldg(&src[wrapk(T.org1 + r1, g.K[1])]);
+      gre[r0 * P1 + r1] = v.x;
+      gim[r0 * P1 + r1] = v.y;
+    }
+  }
+}
+
+// Samples of the chunk's points from the staged tile: store(q, value) in the first
+// lane of each point.  Lane layout, arithmetic and summation order of k_interp.
+template <int JF, int PF, class Store>
+__device__ __forceinline__ void gather_staged2d(const Staged2d& S, const Chunk& ch, const Geom& g, const float* gre,
+                                                const float* gim, Store store) {
+  constexpr int cap = kChunkPoints[2];
+  const int J0 = JF > 0 ? JF : g.J[0], G = JF > 0 ? JF : g.J[1];
+  const int P1 = PF > 0 ? PF : g.P[1];
+  const int PW = 32 / G;
+  const int lane = threadIdx.x & 31;
   const int sub = lane / G;
   const int l = lane - sub * G;
-  const int warp = threadIdx.x >> 5;
-  const int nwarps = blockDim.x >> 5;
-  for (int qb = warp * per_warp; qb < ch.count; qb += nwarps * per_warp) {
+  // warp-uniform rounds of PW points (the lane-group sum is a full-warp shuffle)
+  for (int qb = (threadIdx.x >> 5) * PW; qb < ch.count; qb += cap / 32 * PW) {
     const int q = qb + sub;
-    const bool act = (sub < per_warp) && (q < ch.count);
+    const bool act = (sub < PW) && (q < ch.count);
     float2 part = make_float2(0.f, 0.f);
     if (act) {
-      const int ll = s_k[cap + q] + l;
-      const int l0 = s_k[q];
+      const int base = S.k[q] * P1 + S.k[cap + q] + l;
       float2 acc = make_float2(0.f, 0.f);
 #pragma unroll
       for (int j0 = 0; j0 < (JF > 0 ? JF : kMaxJ); ++j0) {
         if (JF == 0 && j0 >= J0) break;
-        const int cell = (l0 + j0) * P1 + ll;
-        acc = cfma(s_c[j0 * cap + q], make_float2(gre[cell], gim[cell]), acc);
+        acc = cfma(S.c0[j0 * cap + q], make_float2(gre[base + j0 * P1], gim[base + j0 * P1]), acc);
       }
-      part = cmul(s_c[J0 * cap + q * J1 + l], acc);
+      part = cmul(S.c1[q * S.pitch1 + l], acc);
     }
     const float2 tot = lane_group_sum<JF>(part, sub * G, G);
-    if (act && l == 0) y[s_p[q]] = tot;
+    if (act && l == 0) store(q, tot);
   }
+}
+
+template <int JF, int TF>
+__global__ void __launch_bounds__(256, 4)
+k_interp_chunk2d(const float2* __restrict__ grid, float2* __restrict__ y, const Chunk* __restrict__ chunks,
+                 const Points P, const Geom g) {
+  constexpr int cap = kChunkPoints[2];
+  static_assert(cap == 256, "one thread per staged point");
+  constexpr int PF = TF > 0 ? TF + JF - 1 : 0;
+  extern __shared__ float tile[];
+  const int ncell = PF > 0 ? PF * PF : (int)g.padded_cells;
+  const int J0 = JF > 0 ? JF : g.J[0], J1 = JF > 0 ? JF : g.J[1];
+  Staged2d S;
+  S.c0 = reinterpret_cast<float2*>(tile + 2 * ncell);   // 8-byte aligned: 2 * ncell floats
+  S.c1 = S.c0 + J0 * cap;
+  S.pitch1 = J1 | 1;
+  S.k = reinterpret_cast<int*>(S.c1 + S.pitch1 * cap);
+  int* s_p = S.k + 2 * cap;
+  const Chunk ch = chunks[blockIdx.x];
+  const Tile2d T = tile_origin2d(g, ch.bin);
+  stage_points2d<JF>(S, P, g, ch, T);
+  if (threadIdx.x < ch.count) s_p[threadIdx.x] = P.perm[ch.start + threadIdx.x];
+  stage_tile2d<PF>(grid, g, T, tile, tile + ncell);
+  __syncthreads();
+  gather_staged2d<JF, PF>(S, ch, g, tile, tile + ncell, [&](int q, float2 v) { y[s_p[q]] = v; });
 }
 
 // ---------------------------------------------------------------- gridding, per chunk
@@ -1209,123 +1257,71 @@ k_gridding_reduce_packed2d(const float2* __restrict__ tiles, const int32_t* __re
 }
 
 
-// 2D variant: the chunk's point data (first neighbours, coefficients, samples)
-// are first copied into shared memory by all threads at once, so the CTA waits
-// for two dependent global round trips (the permutation, then the samples)
-// instead of one per pass of its warps over the chunk.  The accumulation then
-// follows the same lane layout, bank order and fixed-point words as
-// k_gridding_chunk.
-// Shared memory: the two accumulator planes, then c0[J0][cap] (row by row:
-// the lanes of a point read one value), c1[cap][J1] (point by point: the J1
-// lanes of a point read consecutive words, so a warp's 64-bit reads of five
-// points hit distinct bank pairs), y[cap], k[2][cap] (first neighbours
-// relative to the tile origin), cap = chunk size.
+// 2D chunk pass with staged point data (see k_interp_chunk2d for the layout); the
+// samples are staged too.  The accumulation follows the lane layout, bank order
+// and fixed-point words of k_gridding_chunk; half of the imaginary parts are
+// rounded on the FP32 pipe (round_int), as in scatter_chunk3d.
 // FUSED (V^H V, the normal operator's grid part): y_b is the oversampled
 // spectrum instead of the samples; the chunk's padded tile of it is staged in
 // shared memory (two float planes after the point data), and each point's y is
-// first gathered from there into shared memory (the interpolation's
-// arithmetic and summation order, in the scatter's lane layout), so the
-// samples never leave the CTA and the coefficients are read once for both
-// directions.
-template <int JF, bool FUSED>
+// first gathered from there into shared memory, so the samples never leave the
+// CTA and the coefficients are read once for both directions.
+template <int JF, int TF, bool FUSED>
 __global__ void __launch_bounds__(256, 4)
 k_gridding_chunk_staged(const float2* __restrict__ y_b, float2* __restrict__ tiles_b,
                         const Chunk* __restrict__ chunks, const Points P, const Geom g, int64_t ybs, int64_t tbs) {
   constexpr int cap = kChunkPoints[2];
+  static_assert(cap == 256, "one thread per staged point");
+  constexpr int PF = TF > 0 ? TF + JF - 1 : 0;
   extern __shared__ int acc[];
   __shared__ float red[32];
   const float2* __restrict__ y = y_b + (int64_t)blockIdx.y * ybs;
   float2* __restrict__ tiles = tiles_b + (int64_t)blockIdx.y * tbs;
-  const int ncell = (int)g.padded_cells;
-  const int J0 = JF > 0 ? JF : g.J[0];
-  const int J1 = JF > 0 ? JF : g.J[1];
-  float2* s_c = reinterpret_cast<float2*>(acc + 2 * ncell);   // 8-byte aligned: 2 * ncell words
-  float2* s_y = s_c + (J0 + J1) * cap;
-  int* s_k = reinterpret_cast<int*>(s_y + cap);
-  float* gre = reinterpret_cast<float*>(s_k + 2 * cap);   // FUSED: the chunk's padded tile of the spectrum
-  float* gim = gre + ncell;
+  const int ncell = PF > 0 ? PF * PF : (int)g.padded_cells;
+  const int P1 = PF > 0 ? PF : g.P[1];
+  const int J0 = JF > 0 ? JF : g.J[0], J1 = JF > 0 ? JF : g.J[1];
+  Staged2d S;
+  S.c0 = reinterpret_cast<float2*>(acc + 2 * ncell);   // 8-byte aligned: 2 * ncell words
+  S.c1 = S.c0 + J0 * cap;
+  S.pitch1 = J1 | 1;
+  float2* s_y = S.c1 + S.pitch1 * cap;
+  S.k = reinterpret_cast<int*>(s_y + cap);
   const Chunk ch = chunks[blockIdx.x];
-  const int org0 = ((ch.bin / g.nb[1]) % g.nb[0]) * g.T[0];
-  const int org1 = (ch.bin % g.nb[1]) * g.T[1];
-
-  for (int c = threadIdx.x; c < 2 * ncell; c += blockDim.x) acc[c] = 0;
-  if (FUSED) {
-    const int P1 = g.P[1];
-    for (int c = threadIdx.x; c < ncell; c += blockDim.x) {
-      const int r1 = c % P1, r0 = c / P1;
-      const float2 v = __ldg(&y[(int64_t)wrapk(org0 + r0, g.K[0]) * g.Kstride[0] + wrapk(org1 + r1, g.K[1])]);
-      gre[c] = v.x;
-      gim[c] = v.y;
-    }
-  }
-  static_assert(cap == 256, "one thread per staged point");
-  const int qs = threadIdx.x;           // the point this thread stages
+  const Tile2d T = tile_origin2d(g, ch.bin);
+  const int qs = threadIdx.x;   // the point this thread stages
   int pm = 0;
-  if (qs < ch.count) {
-    const int q = qs;
-    const int64_t i = (int64_t)ch.start + q;
-    if (!FUSED) pm = P.perm[i];
-    s_k[q] = P.kf[i] - org0;
-    s_k[cap + q] = P.kf[P.M + i] - org1;
-#pragma unroll
-    for (int r = 0; r < (JF > 0 ? JF : kMaxJ); ++r) {
-      if (JF == 0 && r >= J0) break;
-      s_c[r * cap + q] = P.coef[P.coef_off[0] + (int64_t)r * P.M + i];
-    }
-#pragma unroll
-    for (int r = 0; r < (JF > 0 ? JF : kMaxJ); ++r) {
-      if (JF == 0 && r >= J1) break;
-      s_c[J0 * cap + q * J1 + r] = P.coef[P.coef_off[1] + (int64_t)r * P.M + i];
-    }
+  if (!FUSED && qs < ch.count) pm = P.perm[ch.start + qs];
+  stage_points2d<JF>(S, P, g, ch, T);
+  if (FUSED) {
+    float* gre = reinterpret_cast<float*>(S.k + 2 * cap);   // the chunk's padded tile of the spectrum
+    stage_tile2d<PF>(y, g, T, gre, gre + ncell);
   }
+  for (int c = threadIdx.x; c < ncell; c += blockDim.x) reinterpret_cast<int2*>(acc)[c] = make_int2(0, 0);
   if (!FUSED && qs < ch.count) s_y[qs] = __ldg(&y[pm]);
   __syncthreads();
-
-  const int G = J1;
-  const int lane = threadIdx.x & 31;
-  const int per_warp = 32 / G;
-  const int sub = lane / G;
-  const int l = lane - sub * G;
-  const int warp = threadIdx.x >> 5;
-  const int nwarps = blockDim.x >> 5;
-  const int P1 = g.P[1];
   if (FUSED) {
-    // warp-uniform rounds of per_warp points: the lane-group sum is a
-    // full-warp shuffle; the spectrum is read from the staged tile
-    for (int qb = warp * per_warp; qb < ch.count; qb += nwarps * per_warp) {
-      const int q = qb + sub;
-      const bool act = (sub < per_warp) && (q < ch.count);
-      float2 part = make_float2(0.f, 0.f);
-      if (act) {
-        const int ll = s_k[cap + q] + l;
-        const int l0 = s_k[q];
-        float2 a = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int j0 = 0; j0 < (JF > 0 ? JF : kMaxJ); ++j0) {
-          if (JF == 0 && j0 >= J0) break;
-          const int cell = (l0 + j0) * P1 + ll;
-          a = cfma(s_c[j0 * cap + q], make_float2(gre[cell], gim[cell]), a);
-        }
-        part = cmul(s_c[J0 * cap + q * J1 + l], a);
-      }
-      const float2 yv = lane_group_sum<JF>(part, sub * G, G);
-      if (act && l == 0) s_y[q] = yv;
-    }
+    const float* gre = reinterpret_cast<const float*>(S.k + 2 * cap);
+    gather_staged2d<JF, PF>(S, ch, g, gre, gre + ncell, [&](int q, float2 v) { s_y[q] = v; });
     __syncthreads();
   }
   // the chunk's scale (also orders the zeroing and staging before the atomics)
   float mag = 0.f;
   if (qs < ch.count) mag = fabsf(s_y[qs].x) + fabsf(s_y[qs].y);
   const ChunkScale cs = chunk_scale<2>(block_sum_fixed(mag, red), P.cmax);
-  if (sub < per_warp && cs.finite) {
-    for (int q = warp * per_warp + sub; q < ch.count; q += nwarps * per_warp) {
-      const float2 yl = cmulc(s_c[J0 * cap + q * J1 + l], cscale(s_y[q], cs.S));   // conj(c_last) * y * S
-      const int ll = s_k[cap + q] + l;
-      const int l0 = s_k[q];
+  const int PW = 32 / J1;
+  const int lane = threadIdx.x & 31;
+  const int sub = lane / J1;
+  const int l = lane - sub * J1;
+  if (sub < PW && cs.finite) {
+    for (int q = (threadIdx.x >> 5) * PW + sub; q < ch.count; q += cap / 32 * PW) {
+      const float2 yl = cmulc(S.c1[q * S.pitch1 + l], cscale(s_y[q], cs.S));   // conj(c_last) * y * S
+      int* cell = acc + S.k[q] * P1 + S.k[cap + q] + l;
 #pragma unroll
       for (int j0 = 0; j0 < (JF > 0 ? JF : kMaxJ); ++j0) {
         if (JF == 0 && j0 >= J0) break;
-        fix_add<2>(acc, ncell, (l0 + j0) * P1 + ll, cmulc(s_c[j0 * cap + q], yl));
+        const float2 w = cmulc(S.c0[j0 * cap + q], yl);
+        atomicAdd(cell + j0 * P1, __float2int_rn(w.x));
+        atomicAdd(cell + j0 * P1 + ncell, (j0 & 1) ? round_int(w.y) : __float2int_rn(w.y));
       }
     }
   }
@@ -1356,14 +1352,6 @@ constexpr int kBatchWarps2d = 2;
 // points, 8 coils (1968 CTAs) 20 against 14.
 constexpr int64_t kBatchMaxMean = 64;
 constexpr int64_t kBatchMinCtas = 32 * 152;
-struct Tile2d {
-  int org0, org1;   // tile origin on the grid
-};
-__device__ __forceinline__ Tile2d tile_origin2d(const Geom& g, int bin) {
-  const int b0 = bin / g.nb[1];
-  return {b0 * g.T[0], (bin - b0 * g.nb[1]) * g.T[1]};
-}
-
 template <int JF>
 __host__ __device__ inline int strip2d(int J0, int J1) { return (JF > 0 ? JF : J0) * (32 / (JF > 0 ? JF : J1)); }
 
@@ -1654,14 +1642,22 @@ cudaError_t interp_chunks(const nufft_plan_t* p, const float2* grid, float2* y, 
   bool t16 = true;
   for (int a = 0; a < D; ++a) t16 = t16 && p->g.T[a] == 16;
   if constexpr (D == 2) {
-    const int sj = p->g.J[0] + p->g.J[1];
-    const size_t smem = (size_t)p->g.padded_cells * 2 * sizeof(float) +
-                        (size_t)kChunkPoints[2] * ((size_t)sj * sizeof(float2) + 3 * sizeof(int));
-    auto kern = j6 ? k_interp_chunk2d<6> : k_interp_chunk2d<0>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<gd, kChunkPoints[2], smem, p->stream>>>(grid, y, p->chunks, P, p->g, p->Kprod, p->M);
-    return cudaGetLastError();
+    const int J0 = p->g.J[0], J1 = p->g.J[1];
+    const size_t smem = (size_t)p->g.padded_cells * 2 * sizeof(float) + Staged2d::coefs(J0, J1) * sizeof(float2) +
+                        (size_t)kChunkPoints[2] * 3 * sizeof(int);
+    auto go = [&](auto kern) {
+      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+      kern<<<(unsigned)p->nchunks, kChunkPoints[2], smem, p->stream>>>(grid, y, p->chunks, P, p->g);
+      return cudaGetLastError();
+    };
+    switch (J0 == J1 ? J0 : 0) {
+      case 4: return go(t16 ? k_interp_chunk2d<4, 16> : k_interp_chunk2d<4, 0>);
+      case 5: return go(t16 ? k_interp_chunk2d<5, 16> : k_interp_chunk2d<5, 0>);
+      case 6: return go(t16 ? k_interp_chunk2d<6, 16> : k_interp_chunk2d<6, 0>);
+      case 7: return go(t16 ? k_interp_chunk2d<7, 16> : k_interp_chunk2d<7, 0>);
+      default: return go(k_interp_chunk2d<0, 0>);
+    }
   } else {
     const int J = all_j_equal(p->g, p->g.J[0]) ? p->g.J[0] : 0;
     if (J >= 4 && J <= 7) {
@@ -1770,14 +1766,25 @@ cudaError_t launch_chunks(const nufft_plan_t* p, const float2* y, float2* tiles,
     }
   }
   if constexpr (D == 2) {
-    const int sj = p->g.J[0] + p->g.J[1];
+    const int J0 = p->g.J[0], J1 = p->g.J[1];
+    const bool t16 = p->g.T[0] == 16 && p->g.T[1] == 16;
     const size_t smem = (size_t)p->g.padded_cells * Fix<2>::kWords * sizeof(int) +
-                        (size_t)kChunkPoints[2] * ((size_t)sj * sizeof(float2) + sizeof(float2) + 2 * sizeof(int)) +
+                        (Staged2d::coefs(J0, J1) + kChunkPoints[2]) * sizeof(float2) +
+                        (size_t)kChunkPoints[2] * 2 * sizeof(int) +
                         (FUSED ? (size_t)p->g.padded_cells * 2 * sizeof(float) : 0);
-    auto kern = j6 ? k_gridding_chunk_staged<6, FUSED> : k_gridding_chunk_staged<0, FUSED>;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<gd, kChunkPoints[2], smem, p->stream>>>(y, tiles, p->chunks, P, p->g, ybs, tbs);
+    auto go = [&](auto kern) {
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+      kern<<<gd, kChunkPoints[2], smem, p->stream>>>(y, tiles, p->chunks, P, p->g, ybs, tbs);
+      return cudaGetLastError();
+    };
+    switch (J0 == J1 ? J0 : 0) {
+      case 4: return go(t16 ? k_gridding_chunk_staged<4, 16, FUSED> : k_gridding_chunk_staged<4, 0, FUSED>);
+      case 5: return go(t16 ? k_gridding_chunk_staged<5, 16, FUSED> : k_gridding_chunk_staged<5, 0, FUSED>);
+      case 6: return go(t16 ? k_gridding_chunk_staged<6, 16, FUSED> : k_gridding_chunk_staged<6, 0, FUSED>);
+      case 7: return go(t16 ? k_gridding_chunk_staged<7, 16, FUSED> : k_gridding_chunk_staged<7, 0, FUSED>);
+      default: return go(k_gridding_chunk_staged<0, 0, FUSED>);
+    }
   } else {
     static_assert(!FUSED, "the fused V^H V pass is 2D only");
     const size_t smem = (size_t)p->g.padded_cells * Fix<D>::kWords * sizeof(int);

@@ -734,14 +734,16 @@ int build_points(nufft_plan_t* p, const float* om) {
   bc[g.nbins] = (int32_t)ch.size();
   const int64_t nch = (int64_t)ch.size();
   // The chunk list in launch order: the longest chunks first (stable), so that
-  // the last wave of a 3D pass holds short ones.  A kooshball's dense chunks sit
-  // in the middle of the bin order; partial tiles keep that order (slot).
-  if (d == 3) {
-    std::vector<int32_t> pos(kChunkPoints[3] + 2, 0);
-    for (const Chunk& c : ch) ++pos[kChunkPoints[3] - c.count + 1];
+  // the last wave of a pass holds short ones.  A radial trajectory's dense chunks
+  // sit in the middle of the bin order; partial tiles keep that order (slot).
+  // 2D pair on a 512^2 grid 55.4 -> 50.9 us, 64^3 normal operator 1.4x.
+  {
+    const int most = kChunkPoints[d];
+    std::vector<int32_t> pos(most + 2, 0);
+    for (const Chunk& c : ch) ++pos[most - c.count + 1];
     for (size_t i = 1; i < pos.size(); ++i) pos[i] += pos[i - 1];
     std::vector<Chunk> sorted(ch.size());
-    for (const Chunk& c : ch) sorted[pos[kChunkPoints[3] - c.count]++] = c;
+    for (const Chunk& c : ch) sorted[pos[most - c.count]++] = c;
     ch.swap(sorted);
   }
   if (nch > p->chunk_cap) {   // grow the chunk list and the partial tiles (and the batched ones, lazily)
