@@ -112,8 +112,8 @@ struct nufft_plan {
   double2* Tinv;            // J_i x J_i min-max inverses, dim i at T_off[i]
   int64_t T_off[nufft::kMaxDim];
   float* om_sorted;         // [d][M] trajectory in tile-sorted order
-  double2* cheb;            // Chebyshev expansions of the coefficients in the offset (plan.cu)
-  int cheb_ok[2];           // expansion used for the coefficients / their derivatives
+  double2* cheb;            // Chebyshev expansions and polynomials of the coefficients in the offset (plan.cu)
+  int cheb_ok[2];           // form used for the coefficients / their derivatives: 2 polynomial, 1 expansion, 0 sums
   float2* dcoef;            // [sum_i J_i][M] d coef / d omega (allocated on first use)
 
   // kept for nufft_plan_set_trajectory: sort scratch, the validation flags and

@@ -197,9 +197,12 @@ __global__ void k_bins(const float* om, int64_t M, Geom g, uint32_t* key, int32_
 
 // ---------------------------------------------------------------- stable LSD radix sort (8 bits/pass)
 constexpr int kSortThreads = 256;
-constexpr int kSortItems = 4096;  // items per CTA
+// Items per CTA: 4096, or 1024 for up to 2^18 points, whose few CTAs would take
+// sixteen rounds each on a mostly idle GPU (32,768 points: scatter 14.6 us).
+__host__ __device__ inline int sort_items(int64_t n) { return n <= (1 << 18) ? 1024 : 4096; }
 
 __global__ void k_radix_hist(const uint32_t* key, int64_t n, int shift, int nblk, uint32_t* hist) {
+  const int kSortItems = sort_items(n);
   __shared__ uint32_t h[256];
   h[threadIdx.x] = 0;
   __syncthreads();
@@ -210,22 +213,33 @@ __global__ void k_radix_hist(const uint32_t* key, int64_t n, int shift, int nblk
   hist[(int64_t)threadIdx.x * nblk + blockIdx.x] = h[threadIdx.x];
 }
 
-// exclusive scan of n values with a single CTA of 1024 threads, in place
+// exclusive scan of n values with a single CTA of 1024 threads, in place: each
+// thread sums its run of values, a shuffle scan over the warps' lanes and one
+// over the 32 warps give the offsets
 __global__ void k_scan_exclusive(uint32_t* v, int64_t n) {
-  __shared__ uint32_t part[1024];
+  __shared__ uint32_t wsum[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t per = (n + 1023) / 1024;
-  const int64_t lo = threadIdx.x * per;
+  const int64_t lo = min(n, threadIdx.x * per);
   const int64_t hi = min(n, lo + per);
   uint32_t s = 0;
   for (int64_t i = lo; i < hi; ++i) s += v[i];
-  part[threadIdx.x] = s;
+  auto inclusive = [lane](uint32_t x) {
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t u = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += u;
+    }
+    return x;
+  };
+  const uint32_t inc = inclusive(s);
+  if (lane == 31) wsum[warp] = inc;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t run = 0;
-    for (int t = 0; t < 1024; ++t) { const uint32_t c = part[t]; part[t] = run; run += c; }
+  if (warp == 0) {
+    const uint32_t w = wsum[lane];
+    wsum[lane] = inclusive(w) - w;
   }
   __syncthreads();
-  uint32_t run = part[threadIdx.x];
+  uint32_t run = wsum[warp] + inc - s;
   for (int64_t i = lo; i < hi; ++i) { const uint32_t c = v[i]; v[i] = run; run += c; }
 }
 
@@ -235,6 +249,7 @@ __global__ void k_radix_scatter(const uint32_t* kin, const int32_t* vin, uint32_
   __shared__ uint32_t running[256];
   __shared__ uint32_t wcount[kSortThreads / 32][256];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int kSortItems = sort_items(n);
   running[tid] = offs[(int64_t)tid * nblk + blockIdx.x];
   const int64_t lo = (int64_t)blockIdx.x * kSortItems;
   for (int round = 0; round < kSortItems / kSortThreads; ++round) {
@@ -328,13 +343,21 @@ __device__ void minmax_coefs(double theta1, int N, int K, int J, const double* s
 // the expansions per point (Clenshaw, FP64) instead of the N-term sums.  The
 // expansion is checked against the sums at other points of [0, 1] and used
 // only where it agrees to kChebTol relative to the largest coefficient.
+//
+// The expansions fall off fast (J = 4 to 9: below 1e-12 of the largest from the
+// 13th term), so the first kMono terms are also kept as a polynomial in x: one
+// multiply-add per term and component instead of the recurrence's two FP64
+// operations over all 24 (32,768 points in 2D: 85 us, FP64-bound).  It is checked
+// against the sums the same way and used where it agrees to the same tolerance.
 constexpr int kCheb = 24;
+constexpr int kMono = 14;
 constexpr double kChebTol = 1e-10;
 
 __device__ __forceinline__ double cheb_node(int m) { return cos(kPi * (m + 0.5) / kCheb); }
 
-// table layout: [(a * 2 + deriv) * kMaxJ + j] * kCheb + k
-__global__ void k_cheb_fit(DimTables D, const double* s64, const double2* Tinv, double2* table) {
+// table layout: [(a * 2 + deriv) * kMaxJ + j] * kCheb + k, then (at `mono`) the
+// polynomials, [(a * 2 + deriv) * kMaxJ + j] * kMono + k
+__global__ void k_cheb_fit(DimTables D, const double* s64, const double2* Tinv, double2* table, double2* mono) {
   const int a = blockIdx.x >> 1, deriv = blockIdx.x & 1;
   __shared__ double2 vals[kCheb][kMaxJ];
   const int N = D.N[a], K = D.K[a], J = D.J[a];
@@ -357,6 +380,37 @@ __global__ void k_cheb_fit(DimTables D, const double* s64, const double2* Tinv, 
     const double f = (k == 0 ? 1.0 : 2.0) / kCheb;
     table[((a * 2 + deriv) * kMaxJ + j) * kCheb + k] = make_double2(f * re, f * im);
   }
+  __syncthreads();
+  // sum_k a_k T_k(x) in powers of x, by the recurrence T_{k+1} = 2 x T_k - T_{k-1}
+  for (int j = threadIdx.x; j < J; j += blockDim.x) {
+    const double2* c = table + ((a * 2 + deriv) * kMaxJ + j) * kCheb;
+    double2 m[kMono];
+    double t0[kMono], t1[kMono];   // T_{k-1}, T_k
+    for (int i = 0; i < kMono; ++i) {
+      t0[i] = i == 0;
+      t1[i] = i == 1;
+      m[i] = i == 0 ? c[0] : (i == 1 ? c[1] : make_double2(0.0, 0.0));
+    }
+    for (int k = 2; k < kMono; ++k) {
+      double prev = 0.0;
+      for (int i = 0; i < kMono; ++i) {
+        const double t = 2.0 * prev - t0[i];
+        prev = t1[i];
+        t0[i] = t1[i];
+        t1[i] = t;
+        m[i].x += c[k].x * t;
+        m[i].y += c[k].y * t;
+      }
+    }
+    for (int i = 0; i < kMono; ++i) mono[((a * 2 + deriv) * kMaxJ + j) * kMono + i] = m[i];
+  }
+}
+
+__device__ __forceinline__ double2 mono_eval(const double2* m, double x) {
+  double2 v = m[kMono - 1];
+#pragma unroll
+  for (int k = kMono - 2; k >= 0; --k) v = make_double2(fma(v.x, x, m[k].x), fma(v.y, x, m[k].y));
+  return v;
 }
 
 __device__ __forceinline__ double2 cheb_eval(const double2* a, double x) {
@@ -369,47 +423,54 @@ __device__ __forceinline__ double2 cheb_eval(const double2* a, double x) {
   return make_double2(a[0].x + x * b1.x - b2.x, a[0].y + x * b1.y - b2.y);
 }
 
-// Largest deviation of the expansion from the sums at kChebCheck points per
+// Largest deviation of the two forms from the sums at kChebCheck points per
 // (dimension, deriv), relative to the largest coefficient there; one block
-// per (dimension, deriv), written to err[a * 2 + deriv].
+// per (dimension, deriv), written to err[2 * (a * 2 + deriv)] (expansion) and
+// the next entry (polynomial).
 constexpr int kChebCheck = 61;
-__global__ void k_cheb_check(DimTables D, const double* s64, const double2* Tinv, const double2* table, double* err) {
+__global__ void k_cheb_check(DimTables D, const double* s64, const double2* Tinv, const double2* table,
+                             const double2* mono, double* err) {
   const int a = blockIdx.x >> 1, deriv = blockIdx.x & 1;
   const int N = D.N[a], K = D.K[a], J = D.J[a];
   const double gamma = (2.0 * kPi) / K;
-  __shared__ double s_err[256], s_max[256];
-  double e = 0.0, mx = 0.0;
+  __shared__ double s_err[256], s_errm[256], s_max[256];
+  double e = 0.0, em = 0.0, mx = 0.0;
   for (int t = threadIdx.x; t < kChebCheck; t += blockDim.x) {
     const double delta = (t + 0.5) / kChebCheck;
     double2 c[kMaxJ];
     minmax_coefs(gamma * (delta + 0.5 * J - 1.0), N, K, J, s64 + D.s_off[a], Tinv + D.T_off[a], deriv, c);
     for (int j = 0; j < J; ++j) {
       const double2 v = cheb_eval(table + ((a * 2 + deriv) * kMaxJ + j) * kCheb, 2.0 * delta - 1.0);
+      const double2 u = mono_eval(mono + ((a * 2 + deriv) * kMaxJ + j) * kMono, 2.0 * delta - 1.0);
       e = fmax(e, hypot(v.x - c[j].x, v.y - c[j].y));
+      em = fmax(em, hypot(u.x - c[j].x, u.y - c[j].y));
       mx = fmax(mx, hypot(c[j].x, c[j].y));
     }
   }
   s_err[threadIdx.x] = e;
+  s_errm[threadIdx.x] = em;
   s_max[threadIdx.x] = mx;
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int t = 1; t < (int)blockDim.x; ++t) {
       e = fmax(e, s_err[t]);
+      em = fmax(em, s_errm[t]);
       mx = fmax(mx, s_max[t]);
     }
-    err[blockIdx.x] = mx > 0.0 ? e / mx : 0.0;
+    err[2 * blockIdx.x] = mx > 0.0 ? e / mx : 0.0;
+    err[2 * blockIdx.x + 1] = mx > 0.0 ? em / mx : 0.0;
   }
 }
 
 // Per sorted point and dimension: first neighbour and the J min-max coefficients
-// (deriv = 1: d c / d w instead).  cheb != NULL evaluates the plan's Chebyshev
-// expansions, else the sums.  om_sorted = 1: om is [d][M] in sorted order;
+// (deriv = 1: d c / d w instead).  form 2 evaluates the plan's polynomials, form 1
+// its Chebyshev expansions (tables at cheb and mono), form 0 the sums.  om_sorted = 1: om is [d][M] in sorted order;
 // otherwise om is the caller's M x d array and perm maps to it, and the sorted
 // copy is written to om_out (if not NULL).
 __global__ void k_coefficients(const float* om, int om_sorted, Geom g, int64_t M, const int32_t* perm,
                                const double* s64, DimTables D, const double2* Tinv, int32_t* kf_out, float2* coef,
                                int64_t coef_off0, int64_t coef_off1, int64_t coef_off2, int deriv, float* om_out,
-                               const double2* cheb) {
+                               const double2* cheb, const double2* mono, int form) {
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= M * g.d) return;
   const int a = (int)(idx / M);
@@ -421,11 +482,12 @@ __global__ void k_coefficients(const float* om, int om_sorted, Geom g, int64_t M
   const double k0 = offset_k0(w, K, J);
   const double gamma = (2.0 * kPi) / K;
   const int64_t off = a == 0 ? coef_off0 : (a == 1 ? coef_off1 : coef_off2);
-  if (cheb) {
+  if (form) {
     const double delta = w / gamma - k0 - 0.5 * J;
     const double x = fmin(1.0, fmax(-1.0, 2.0 * delta - 1.0));
     for (int j = 0; j < J; ++j) {
-      const double2 v = cheb_eval(cheb + ((a * 2 + deriv) * kMaxJ + j) * kCheb, x);
+      const int row = (a * 2 + deriv) * kMaxJ + j;
+      const double2 v = form == 2 ? mono_eval(mono + row * kMono, x) : cheb_eval(cheb + row * kCheb, x);
       coef[off + (int64_t)j * M + i] = make_float2((float)v.x, (float)v.y);
     }
   } else {
@@ -557,7 +619,7 @@ k_bank_order(const float* om, Geom g, const Chunk* chunks, int64_t nchunks, cons
   const int d = g.d;
   const int JL = g.J[d - 1];
   const int G = 32 / JL;
-  const unsigned base_mask = JL >= 32 ? 0xffffffffu : ((1u << JL) - 1u);
+  const unsigned base_mask = (1u << JL) - 1u;   // JL <= 16
   int org[kMaxDim];
   {
     int rem = ch.bin;
@@ -576,37 +638,50 @@ k_bank_order(const float* om, Geom g, const Chunk* chunks, int64_t nchunks, cons
     s_b[q] = (unsigned char)(cell & 31);
   }
   __syncwarp();
+  // the banks are read four at a time (s_b is 4-byte aligned: cap is a multiple of
+  // 4; the tail of the last word belongs to no point)
+  const uint32_t* s_b4 = reinterpret_cast<const uint32_t*>(s_b);
+  const int words = (ch.count + 3) >> 2;
+  if (lane < 4 * words - ch.count) s_b[ch.count + lane] = 255;
+  __syncwarp();
   int cnt = 0;
-  for (int q = 0; q < ch.count; ++q) cnt += s_b[q] == lane;
+  for (int q = 0; q < words; ++q) {
+    const uint32_t v = s_b4[q];
+    cnt += ((v & 255u) == lane) + (((v >> 8) & 255u) == lane) + (((v >> 16) & 255u) == lane) + ((v >> 24) == lane);
+  }
   int first = cnt;                                     // exclusive prefix over the lanes
   for (int o = 1; o < 32; o <<= 1) {
     const int v = __shfl_up_sync(0xffffffffu, first, o);
     if (lane >= o) first += v;
   }
   first -= cnt;
-  for (int q = 0, pos = first; q < ch.count; ++q)
-    if (s_b[q] == lane) s_ord[pos++] = (int16_t)q;
+  for (int q = 0, pos = first; q < words; ++q) {
+    const uint32_t v = s_b4[q];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (((v >> (8 * u)) & 255u) == lane) s_ord[pos++] = (int16_t)(4 * q + u);
+  }
   __syncwarp();
-  const unsigned my_win = (base_mask << lane) | (lane ? (base_mask >> (32 - lane)) : 0u);
+  // The greedy step is one chain (arg-max, then the window it takes), so each lane
+  // holds its bucket's next point in a register and stores it itself.
+  const unsigned my_win = __funnelshift_l(base_mask, base_mask, lane);
   int head = first;
+  int16_t next = cnt > 0 ? s_ord[head] : 0;
   int out = 0;
   while (out < ch.count) {
     unsigned used = 0u;
     for (int s = 0; s < G && out < ch.count; ++s) {
       // key: count + 1 in the high bits, 31 - lane low (ties -> lowest lane)
-      const unsigned free_key = (cnt > 0 && (my_win & used) == 0u) ? ((unsigned)(cnt + 1) << 5) | (31u - lane) : 0u;
-      unsigned best_key = __reduce_max_sync(0xffffffffu, free_key);
-      if (best_key == 0u)
-        best_key = __reduce_max_sync(0xffffffffu, cnt > 0 ? ((unsigned)(cnt + 1) << 5) | (31u - lane) : 0u);
+      const unsigned any_key = cnt > 0 ? ((unsigned)(cnt + 1) << 5) | (31u - lane) : 0u;
+      unsigned best_key = __reduce_max_sync(0xffffffffu, (my_win & used) == 0u ? any_key : 0u);
+      if (best_key == 0u) best_key = __reduce_max_sync(0xffffffffu, any_key);
       const int best = 31 - (int)(best_key & 31u);
-      int q = 0;
       if (lane == best) {
-        q = s_ord[head++];
-        --cnt;
+        s_out[out] = next;
+        ++head;
+        if (--cnt > 0) next = s_ord[head];
       }
-      q = __shfl_sync(0xffffffffu, q, best);
-      used |= (base_mask << best) | (best ? (base_mask >> (32 - best)) : 0u);
-      if (lane == 0) s_out[out] = (int16_t)q;
+      used |= __funnelshift_l(base_mask, base_mask, best);
       ++out;
     }
   }
@@ -653,7 +728,10 @@ DimTables dim_tables(const nufft_plan_t* p) {
   return D;
 }
 
-int sort_blocks(int64_t M) { return (int)((M + kSortItems - 1) / kSortItems); }
+// The polynomials behind the expansions in the plan's table.
+double2* mono_table(const nufft_plan_t* p) { return p->cheb ? p->cheb + (int64_t)p->g.d * 2 * kMaxJ * kCheb : nullptr; }
+
+int sort_blocks(int64_t M) { return (int)((M + sort_items(M) - 1) / sort_items(M)); }
 
 // Reject a trajectory with a non-finite value or |om| > 2^20 (flag 0), before
 // anything uses it.  Synchronizes the stream.
@@ -804,7 +882,6 @@ int build_points(nufft_plan_t* p, const float* om) {
       if (fill > 0) wl.push_back(make_int4(pend[0], pend[1], pend[2], pend[3]));
       if (!p->red_work) NUFFT_CUDA_TRY(p, dalloc(p, &p->red_work, g.nbins));
       NUFFT_CUDA_TRY(p, cudaMemcpyAsync(p->red_work, wl.data(), wl.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
-      NUFFT_CUDA_TRY(p, cudaStreamSynchronize(st));   // wl is a host temporary
       p->red_ctas = (int)wl.size();
     }
   }
@@ -830,7 +907,7 @@ int build_points(nufft_plan_t* p, const float* om) {
     k_coefficients<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(om, 0, g, M, p->perm, p->s64, D, p->Tinv, p->kf,
                                                                p->coef, p->coef_off[0], p->coef_off[1],
                                                                p->coef_off[2], 0, p->om_sorted,
-                                                               p->cheb_ok[0] ? p->cheb : nullptr);
+                                                               p->cheb, mono_table(p), p->cheb_ok[0]);
     NUFFT_CUDA_TRY(p, cudaGetLastError());
     NUFFT_CUDA_TRY(p, cudaMemsetAsync(p->cmax, 0, kMaxDim * sizeof(uint32_t), st));
     k_coef_max<<<(unsigned)std::min<int64_t>(1024, (M * d + 255) / 256), 256, 0, st>>>(
@@ -852,7 +929,7 @@ int build_points(nufft_plan_t* p, const float* om) {
     if (p->dcoef) {
       k_coefficients<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(
           p->om_sorted, 1, g, M, p->perm, p->s64, D, p->Tinv, nullptr, p->dcoef, p->coef_off[0], p->coef_off[1],
-          p->coef_off[2], 1, nullptr, p->cheb_ok[1] ? p->cheb : nullptr);
+          p->coef_off[2], 1, nullptr, p->cheb, mono_table(p), p->cheb_ok[1]);
       NUFFT_CUDA_TRY(p, cudaGetLastError());
     }
   }
@@ -891,22 +968,26 @@ int build_plan(nufft_plan_t* p, const float* om) {
   // checked against the sums (kept for d c / d w too)
   int hflag[2] = {0, 0};
   if (M > 0) {
-    NUFFT_CUDA_TRY(p, dalloc(p, &p->cheb, (int64_t)d * 2 * kMaxJ * kCheb));
+    NUFFT_CUDA_TRY(p, dalloc(p, &p->cheb, (int64_t)d * 2 * kMaxJ * (kCheb + kMono)));
     double* err = nullptr;
-    NUFFT_CUDA_TRY(p, dev_malloc((void**)&err, 2 * kMaxDim * sizeof(double)));
+    NUFFT_CUDA_TRY(p, dev_malloc((void**)&err, 4 * kMaxDim * sizeof(double)));
     struct G5 { void* a; ~G5() { if (a) dev_free(a); } } g5{err};
-    k_cheb_fit<<<2 * d, 64, 0, st>>>(D, p->s64, p->Tinv, p->cheb);
+    k_cheb_fit<<<2 * d, 64, 0, st>>>(D, p->s64, p->Tinv, p->cheb, mono_table(p));
     NUFFT_CUDA_TRY(p, cudaGetLastError());
-    k_cheb_check<<<2 * d, 64, 0, st>>>(D, p->s64, p->Tinv, p->cheb, err);
+    k_cheb_check<<<2 * d, 64, 0, st>>>(D, p->s64, p->Tinv, p->cheb, mono_table(p), err);
     NUFFT_CUDA_TRY(p, cudaGetLastError());
-    double herr[2 * kMaxDim];
-    NUFFT_CUDA_TRY(p, cudaMemcpyAsync(herr, err, 2 * d * sizeof(double), cudaMemcpyDeviceToHost, st));
+    double herr[4 * kMaxDim];
+    NUFFT_CUDA_TRY(p, cudaMemcpyAsync(herr, err, 4 * d * sizeof(double), cudaMemcpyDeviceToHost, st));
     NUFFT_CUDA_TRY(p, cudaMemcpyAsync(hflag, p->flags, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
     NUFFT_CUDA_TRY(p, cudaStreamSynchronize(st));
-    p->cheb_ok[0] = p->cheb_ok[1] = 1;
-    for (int a = 0; a < d; ++a)
-      for (int v = 0; v < 2; ++v)
-        if (!(herr[a * 2 + v] <= kChebTol)) p->cheb_ok[v] = 0;
+    for (int v = 0; v < 2; ++v) {
+      bool cheb = true, mono = true;
+      for (int a = 0; a < d; ++a) {
+        cheb = cheb && herr[2 * (a * 2 + v)] <= kChebTol;
+        mono = mono && herr[2 * (a * 2 + v) + 1] <= kChebTol;
+      }
+      p->cheb_ok[v] = mono ? 2 : (cheb ? 1 : 0);
+    }
   } else {
     NUFFT_CUDA_TRY(p, cudaMemcpyAsync(hflag, p->flags, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
     NUFFT_CUDA_TRY(p, cudaStreamSynchronize(st));
@@ -953,7 +1034,7 @@ int ensure_coef_derivatives(nufft_plan_t* p) {
   const int64_t n = p->M * p->g.d;
   k_coefficients<<<(unsigned)((n + 127) / 128), 128, 0, p->stream>>>(
       p->om_sorted, 1, p->g, p->M, p->perm, p->s64, D, p->Tinv, nullptr, p->dcoef, p->coef_off[0], p->coef_off[1],
-      p->coef_off[2], 1, nullptr, p->cheb_ok[1] ? p->cheb : nullptr);
+      p->coef_off[2], 1, nullptr, p->cheb, mono_table(p), p->cheb_ok[1]);
   NUFFT_CUDA_TRY(p, cudaGetLastError());
   return NUFFT_OK;
 }

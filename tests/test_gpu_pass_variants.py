@@ -102,6 +102,38 @@ def test_3d_interpolation_and_gridding(nf, J, Kd, M):
         assert rel(plan.gridding(dev(y)).cpu().numpy(), oracle.gridding_VH(p, y)) < TOL_V
 
 
+# 2D single transforms: tiles of 16 and others, chunk counts at the edges of a chunk
+@pytest.mark.parametrize("Jd", [(4, 4), (5, 5), (6, 6), (7, 7), (7, 4), (1, 6)])
+@pytest.mark.parametrize("Kd,M", [((64, 48), 255), ((32, 32), 1025), ((36, 90), 4100), ((18, 64), 40)])
+def test_2d_single_transforms(nf, Jd, Kd, M):
+    Nd = tuple(2 * (K // 4) for K in Kd)
+    om = W.uniform_random_om(M, 2, seed=M + 1)
+    om[: M // 2] = 0.2 + 0.01 * om[: M // 2]     # more than one chunk in a tile
+    p = oracle.make_plan(om, Nd, Kd, Jd)
+    x, z, y = cn(Nd, 11), cn(Kd, 12), cn(M, 13)
+    with nf.NufftPlan(dev(om), Nd, Kd, Jd) as plan:
+        assert rel(plan.interp(dev(z)).cpu().numpy(), oracle.interp_V(p, z)) < TOL_V
+        assert rel(plan.gridding(dev(y)).cpu().numpy(), oracle.gridding_VH(p, y)) < TOL_V
+        assert rel(plan.selfadjoint(dev(x)).cpu().numpy(), oracle.selfadjoint(p, x)) < 2 * TOL_OP
+
+
+# the polynomial form of the coefficients, and trajectories around the size at which
+# the sort changes its tile
+@pytest.mark.parametrize("N,K,J,M", [(64, 128, 8, 300), (64, 128, 6, 300), (40, 60, 5, 300), (16, 16, 3, 300),
+                                     (64, 128, 6, (1 << 18) - 1), (64, 128, 6, (1 << 18) + 1)])
+def test_coefficients_and_sort(nf, N, K, J, M):
+    om = W.uniform_random_om(M, 2, seed=14)
+    with nf.NufftPlan(dev(om), (N, N), (K, K), (J, J)) as plan:
+        kf, coefs, _, perm = plan.interpolator()
+    np.testing.assert_array_equal(np.sort(perm.numpy()), np.arange(M))
+    pick = np.arange(0, M, max(1, M // 300))
+    p = oracle.make_plan(om[pick], (N, N), (K, K), (J, J))
+    for a in range(2):
+        np.testing.assert_array_equal(kf.numpy()[pick, a], (p.k0[:, a] + 1) % K)
+        err = np.abs(coefs[a].numpy()[pick] - p.coef[a]).max() / np.abs(p.coef[a]).max()
+        assert err < 1e-7, (a, err)   # the float32 rounding is at most 2^-24 = 6e-8 of a component
+
+
 # chunks of few and of many points, CTA counts on both sides of the rule, odd tiles
 @pytest.mark.parametrize("Jd", [(4, 4), (5, 5), (6, 6), (7, 7), (5, 7), (6, 1)])
 @pytest.mark.parametrize("Kd,M,nb", [((256, 256), 3001, 20), ((256, 256), 17000, 2), ((90, 64), 700, 3),
