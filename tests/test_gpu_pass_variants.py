@@ -51,7 +51,7 @@ def dev(a):
     ((128, 96, 64), (64, 48, 32)), ((256, 48, 64), (200, 24, 32)), ((128, 64, 64), (64, 32, 32)),
     ((64, 128, 128), (64, 64, 100)), ((64, 256, 64), (50, 128, 64)), ((128, 90, 90), (64, 60, 90)),
     ((256, 50, 30), (128, 26, 30)), ((16, 32, 1024), (16, 20, 512)), ((512, 128), (256, 128)), ((1024, 36), (512, 18)),
-    ((64, 512), (34, 512)),
+    ((64, 512), (34, 512)), ((512, 36, 36), (256, 18, 36)),
 ])
 def test_fft_passes(nf, Kd, Nd):
     d = len(Kd)
