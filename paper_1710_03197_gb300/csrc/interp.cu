@@ -174,7 +174,7 @@ k_interp(const float2* __restrict__ grid_b, float2* __restrict__ y_b, const Poin
 }
 
 // ---------------------------------------------------------------- interpolation, per chunk
-// One CTA per chunk of a tile's points (3D; 2D below).  The chunk's padded tile of
+// One CTA per chunk of a tile's points.  The chunk's padded tile of
 // the grid ((T+J-1)^d cells, wrapped at the grid edge) is copied into shared
 // memory once, as a plane of real parts and a plane of imaginary parts, and
 // every point gathers its J^d neighbours from there instead of from global
@@ -183,63 +183,42 @@ k_interp(const float2* __restrict__ grid_b, float2* __restrict__ y_b, const Poin
 // the same order for its atomics).  Lane layout, arithmetic and summation
 // order are those of k_interp (results agree to rounding: the compiler may
 // fuse the multiply-adds differently in the two kernels).
-template <int D>
-struct InterpChunkCfg {
-  static constexpr int kThreads = D == 3 ? 512 : 256;
-  static constexpr int kMinBlocks = D == 3 ? 2 : 4;
-};
 
-template <int D, int JF, int TF>
-__global__ void __launch_bounds__(InterpChunkCfg<D>::kThreads, InterpChunkCfg<D>::kMinBlocks)
-k_interp_chunk(const float2* __restrict__ grid_b, float2* __restrict__ y_b, const Chunk* __restrict__ chunks,
-               const Points P, const Geom g, int64_t gbs, int64_t ybs) {
-  static_assert(TF == 0 || JF > 0, "a fixed tile needs a fixed J");
-  constexpr int PF = TF > 0 ? TF + JF - 1 : 0;
+// 3D, any J (k_interp_chunk3d takes equal J from 4 to 7).
+__global__ void __launch_bounds__(512, 2)
+k_interp_chunk3d_any(const float2* __restrict__ grid, float2* __restrict__ y, const Chunk* __restrict__ chunks,
+                     const Points P, const Geom g) {
   extern __shared__ float tile[];
-  const float2* __restrict__ grid = grid_b + (int64_t)blockIdx.y * gbs;
-  float2* __restrict__ y = y_b + (int64_t)blockIdx.y * ybs;
-  const int ncell = TF > 0 ? (D == 2 ? PF * PF : PF * PF * PF) : (int)g.padded_cells;
-  const int P1 = TF > 0 ? PF : g.P[1];
-  const int P2 = D > 2 ? (TF > 0 ? PF : g.P[2]) : 1;
+  const int ncell = (int)g.padded_cells;
+  const int P1 = g.P[1], P2 = g.P[2];
   float* gre = tile;
   float* gim = tile + ncell;
   const Chunk ch = chunks[blockIdx.x];
-  int org[kMaxDim];
+  int org[3];
   {
     int rem = ch.bin;
-    for (int a = D - 1; a >= 0; --a) {
+    for (int a = 2; a >= 0; --a) {
       org[a] = (rem % g.nb[a]) * g.T[a];
       rem /= g.nb[a];
     }
   }
-  // the padded tile, cell c = (r0, r1[, r2]) in C order with pitches P
+  // the padded tile, cell c = (r0, r1, r2) in C order with pitches P
   for (int c = threadIdx.x; c < ncell; c += blockDim.x) {
-    int r0, r1, r2 = 0;
-    if (D == 2) {
-      r1 = c % P1;
-      r0 = c / P1;
-    } else {
-      r2 = c % P2;
-      r1 = (c / P2) % P1;
-      r0 = c / (P2 * P1);
-    }
-    int64_t gi = (int64_t)wrapk(org[0] + r0, g.K[0]) * g.Kstride[0] + (int64_t)wrapk(org[1] + r1, g.K[1]) * g.Kstride[1];
-    if (D == 3) gi += wrapk(org[2] + r2, g.K[2]);
-    const float2 v = __ldg(&grid[gi]);
+    const int r2 = c % P2, r1 = (c / P2) % P1, r0 = c / (P2 * P1);
+    const float2 v = __ldg(&grid[wrapk(org[0] + r0, g.K[0]) * (int)g.Kstride[0] +
+                                 wrapk(org[1] + r1, g.K[1]) * (int)g.Kstride[1] + wrapk(org[2] + r2, g.K[2])]);
     gre[c] = v.x;
     gim[c] = v.y;
   }
   __syncthreads();
 
-  const int G = JF > 0 ? JF : g.J[D - 1];
+  const int G = g.J[2], J0 = g.J[0], J1 = g.J[1];
   const int lane = threadIdx.x & 31;
   const int per_warp = 32 / G;
   const int sub = lane / G;
   const int l = lane - sub * G;
   const int warp = threadIdx.x >> 5;
   const int nwarps = blockDim.x >> 5;
-  const int J0 = JF > 0 ? JF : g.J[0];
-  const int J1 = JF > 0 ? JF : (D > 2 ? g.J[1] : 1);
   // warp-uniform rounds of per_warp points (the lane-group sum is a full-warp shuffle)
   for (int qb = warp * per_warp; qb < ch.count; qb += nwarps * per_warp) {
     const int q = qb + sub;
@@ -247,44 +226,32 @@ k_interp_chunk(const float2* __restrict__ grid_b, float2* __restrict__ y_b, cons
     const int64_t i = (int64_t)ch.start + q;
     float2 part = make_float2(0.f, 0.f);
     if (act) {
-      const int ll = P.kf[(int64_t)(D - 1) * P.M + i] - org[D - 1] + l;
-      const float2 cl = P.coef[P.coef_off[D - 1] + (int64_t)l * P.M + i];
-      const int l0 = P.kf[i] - org[0];
+      const int ll = P.kf[2 * P.M + i] - org[2] + l;
+      const float2 cl = P.coef[P.coef_off[2] + (int64_t)l * P.M + i];
+      const int l0 = P.kf[i] - org[0], l1 = P.kf[P.M + i] - org[1];
       float2 acc = make_float2(0.f, 0.f);
-      if (D == 2) {
+      float2 c1v[kMaxJ];
 #pragma unroll
-        for (int j0 = 0; j0 < (JF > 0 ? JF : kMaxJ); ++j0) {
-          if (JF == 0 && j0 >= J0) break;
-          const float2 c0 = P.coef[P.coef_off[0] + (int64_t)j0 * P.M + i];
-          const int cell = (l0 + j0) * P1 + ll;
-          acc = cfma(c0, make_float2(gre[cell], gim[cell]), acc);
-        }
-      } else {
-        const int l1 = P.kf[P.M + i] - org[1];
-        float2 c1v[JF > 0 ? JF : kMaxJ];
+      for (int j1 = 0; j1 < kMaxJ; ++j1) {
+        if (j1 >= J1) break;
+        c1v[j1] = P.coef[P.coef_off[1] + (int64_t)j1 * P.M + i];
+      }
+#pragma unroll 1
+      for (int j0 = 0; j0 < J0; ++j0) {
+        const float2 c0 = P.coef[P.coef_off[0] + (int64_t)j0 * P.M + i];
+        const int rowbase = ((l0 + j0) * P1 + l1) * P2 + ll;
+        float2 acc1 = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int j1 = 0; j1 < (JF > 0 ? JF : kMaxJ); ++j1) {
-          if (JF == 0 && j1 >= J1) break;
-          c1v[j1] = P.coef[P.coef_off[1] + (int64_t)j1 * P.M + i];
+        for (int j1 = 0; j1 < kMaxJ; ++j1) {
+          if (j1 >= J1) break;
+          const int cell = rowbase + j1 * P2;
+          acc1 = cfma(c1v[j1], make_float2(gre[cell], gim[cell]), acc1);
         }
-        constexpr int kU0 = TF > 0 ? JF : 1;
-#pragma unroll kU0
-        for (int j0 = 0; j0 < J0; ++j0) {
-          const float2 c0 = P.coef[P.coef_off[0] + (int64_t)j0 * P.M + i];
-          const int rowbase = ((l0 + j0) * P1 + l1) * P2 + ll;
-          float2 acc1 = make_float2(0.f, 0.f);
-#pragma unroll
-          for (int j1 = 0; j1 < (JF > 0 ? JF : kMaxJ); ++j1) {
-            if (JF == 0 && j1 >= J1) break;
-            const int cell = rowbase + j1 * P2;
-            acc1 = cfma(c1v[j1], make_float2(gre[cell], gim[cell]), acc1);
-          }
-          acc = cfma(c0, acc1, acc);
-        }
+        acc = cfma(c0, acc1, acc);
       }
       part = cmul(cl, acc);
     }
-    const float2 tot = lane_group_sum<JF>(part, sub * G, G);
+    const float2 tot = lane_group_sum<0>(part, sub * G, G);
     if (act && l == 0) y[P.perm[i]] = tot;
   }
 }
@@ -1016,8 +983,6 @@ k_gridding_chunk(const float2* __restrict__ y_b, float2* __restrict__ tiles_b, c
 // source bin's chunks, in a fixed order.
 // The whole CTA reduces grid tile `bin`; `part` is shared scratch of
 // blockDim.x * CPT values.
-// The cells reduced are cbase .. cbase + (blockDim/NG)*CPT - 1 of the tile (all
-// of it when cbase = 0 and the groups span it).
 // Entry n (2^D bits at bit 2^D * n) is the set of the e in [0, 2^D) with
 // e & ~n == 0: the neighbours whose padded tiles reach a cell that is near the
 // low edge of its tile along the axes in n.
@@ -1031,11 +996,11 @@ __host__ __device__ constexpr uint64_t subset_masks() {
 }
 
 // Per-cell set-up of a tile reduction: the thread's CPT cells are
-// cbase + tg + k * gsize of tile bc (coordinates in tiles); loc0 is a cell's
+// tg + k * gsize of tile bc (coordinates in tiles); loc0 is a cell's
 // offset in a padded tile, emask the neighbours e whose padded tiles reach it
 // (0 beyond cend), goff its grid offset.
 template <int D, int CPT, int TF>
-__device__ __forceinline__ void reduce_cells(const Geom& g, const int (&bc)[kMaxDim], int cbase, int tg, int gsize,
+__device__ __forceinline__ void reduce_cells(const Geom& g, const int (&bc)[kMaxDim], int tg, int gsize,
                                              int tile_cells, int cend, int (&loc0)[CPT], unsigned (&emask)[CPT],
                                              int (&goff)[CPT]) {
   const int P1 = D > 1 ? g.P[1] : 1, P2 = D > 2 ? g.P[2] : 1;
@@ -1043,7 +1008,7 @@ __device__ __forceinline__ void reduce_cells(const Geom& g, const int (&bc)[kMax
   const int T1 = D > 1 ? (TF > 0 ? TF : g.T[1]) : 1, T2 = D > 2 ? (TF > 0 ? TF : g.T[2]) : 1;
 #pragma unroll
   for (int k = 0; k < CPT; ++k) {
-    const int c = min(cbase + tg + k * gsize, tile_cells - 1);
+    const int c = min(tg + k * gsize, tile_cells - 1);
     int lc[3] = {0, 0, 0};
     if (D == 1) {
       lc[0] = c;
@@ -1063,7 +1028,7 @@ __device__ __forceinline__ void reduce_cells(const Geom& g, const int (&bc)[kMax
 #pragma unroll
     for (int a = 0; a < D; ++a) near |= (lc[a] + g.T[a] < g.P[a] ? 1u : 0u) << (D - 1 - a);
     const unsigned m = (unsigned)(subset_masks<D>() >> ((1 << D) * near)) & ((1u << (1 << D)) - 1u);
-    emask[k] = (cbase + tg + k * gsize < cend) ? m : 0u;
+    emask[k] = (tg + k * gsize < cend) ? m : 0u;
     int off = 0;
 #pragma unroll
     for (int a = 0; a < D; ++a) off += (bc[a] * g.T[a] + lc[a]) * (int)g.Kstride[a];
@@ -1074,7 +1039,7 @@ __device__ __forceinline__ void reduce_cells(const Geom& g, const int (&bc)[kMax
 template <int D, int CPT, int TF>
 __device__ __forceinline__ void reduce_tile(const float2* __restrict__ tiles, const int32_t* __restrict__ bin_chunk,
                                             float2* __restrict__ grid, const Geom& g, const int NG, const int bin,
-                                            float2* part, const int cbase = 0) {
+                                            float2* part) {
   // NG thread groups of blockDim/NG threads; group h takes every NG-th (e, chunk)
   // pair, and the groups' sums are added in group order at the end.
   __shared__ int s_q0[1 << kMaxDim], s_q1[1 << kMaxDim], s_delta[1 << kMaxDim];
@@ -1117,10 +1082,10 @@ __device__ __forceinline__ void reduce_tile(const float2* __restrict__ tiles, co
   for (int e = 0; e < (1 << D); ++e) npairs += s_q1[e] - s_q0[e];
   const int NGe = npairs > 2 * (1 << D) ? NG : 1;
   const bool active = h < NGe;
-  const int cend = min(tile_cells, cbase + gsize * CPT);
+  const int cend = min(tile_cells, gsize * CPT);
 #pragma unroll
   for (int k = 0; k < CPT; ++k) acc[k] = make_float2(0.f, 0.f);
-  reduce_cells<D, CPT, TF>(g, bc, cbase, tg, gsize, tile_cells, cend, loc0, emask, goff);
+  reduce_cells<D, CPT, TF>(g, bc, tg, gsize, tile_cells, cend, loc0, emask, goff);
   const int64_t pc = g.padded_cells;
   if (active) {
     int idx = 0;  // running index over the (e, chunk) pairs
@@ -1176,7 +1141,7 @@ __device__ __forceinline__ void reduce_tile(const float2* __restrict__ tiles, co
   if (h == 0) {
 #pragma unroll
     for (int k = 0; k < CPT; ++k)
-      if (cbase + tg + k * gsize < cend) grid[goff[k]] = acc[k];
+      if (tg + k * gsize < cend) grid[goff[k]] = acc[k];
   }
   __syncthreads();   // shared scratch free for the caller
 }
@@ -1218,7 +1183,7 @@ __device__ __forceinline__ void reduce_tile_group2d(const float2* __restrict__ t
   float2 acc[CPT];
 #pragma unroll
   for (int k = 0; k < CPT; ++k) acc[k] = make_float2(0.f, 0.f);
-  reduce_cells<2, CPT, TF>(g, bc, 0, tg, gsize, tile_cells, cend, loc0, emask, goff);
+  reduce_cells<2, CPT, TF>(g, bc, tg, gsize, tile_cells, cend, loc0, emask, goff);
   const int64_t pc = g.padded_cells;
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
@@ -1246,7 +1211,7 @@ k_gridding_reduce_packed2d(const float2* __restrict__ tiles, const int32_t* __re
   extern __shared__ float2 part[];
   const int4 w = work[blockIdx.x];
   if (w.y == -2) {   // CTA-uniform
-    reduce_tile<2, CPT, TF>(tiles, bin_chunk, grid, g, NG, w.x, part, 0);
+    reduce_tile<2, CPT, TF>(tiles, bin_chunk, grid, g, NG, w.x, part);
     return;
   }
   const int gsize = blockDim.x / NG;
@@ -1676,21 +1641,34 @@ cudaError_t interp_chunks(const nufft_plan_t* p, const float2* grid, float2* y, 
       }
     }
     const size_t smem = (size_t)p->g.padded_cells * 2 * sizeof(float);
-    auto kern = k_interp_chunk<D, 0, 0>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_interp_chunk3d_any, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<gd, InterpChunkCfg<D>::kThreads, smem, p->stream>>>(grid, y, p->chunks, P, p->g, p->Kprod, p->M);
+    k_interp_chunk3d_any<<<(unsigned)p->nchunks, 512, smem, p->stream>>>(grid, y, p->chunks, P, p->g);
     return cudaGetLastError();
   }
 }
 
+// 3D: CTAs from which the staged chunks beat the per-point kernel.  Measured, staged
+// against per point: 27 CTAs (9600 points) 43 us against 11, 200 (115,200) 46
+// against 32, 459 (307,200, with its gridding and FFTs) 176 against 217, 3044 (the
+// 128^3 pair) 855 against 1125; batches: 600 115 against 105, 1152 147 against
+// 148, 1600 234 against 267.
+constexpr int64_t kChunkCtas3d = 304, kChunkCtas3dBatch = 1024;
+
 template <int D>
 cudaError_t interp_d(const nufft_plan_t* p, const float2* grid, float2* y, int nb) {
-  // single transforms gather from staged tiles; a batch keeps the per-point
-  // kernel (the chunk kernel would stage each chunk's point data once per
-  // batch element: the 32-coil frames' normal operator measured 2.36 -> 2.87 ms)
-  if constexpr (D > 1) {
+  // 2D: single transforms gather from staged tiles, batches per point (the chunk
+  // kernel would stage each chunk's point data once per batch element: the
+  // 32-coil frames' normal operator 2.36 -> 2.87 ms).
+  // 3D: staged tiles where the chunks (times batch elements) give the GPU CTAs
+  // enough; fewer are bound by the longest chunk's rounds.
+  if constexpr (D == 2) {
     if (nb == 1) return interp_chunks<D>(p, grid, y, nb);
+  }
+  if constexpr (D == 3) {
+    const int J = all_j_equal(p->g, p->g.J[0]) ? p->g.J[0] : 0;
+    if (J >= 4 && J <= 7 ? p->nchunks * nb >= (nb == 1 ? kChunkCtas3d : kChunkCtas3dBatch) : nb == 1)
+      return interp_chunks<D>(p, grid, y, nb);
   }
   const Points P = points_view(p);
   const int G = p->g.J[D - 1];
@@ -1712,7 +1690,15 @@ cudaError_t interp_d(const nufft_plan_t* p, const float2* grid, float2* y, int n
     }
   }
   const dim3 gd((unsigned)blocks, (unsigned)nb);
-  auto kern = D != 2 && all_j_equal(p->g, 6) ? k_interp<D, (D != 2 ? 6 : 0)> : k_interp<D, 0>;
+  auto kern = k_interp<D, 0>;
+  if constexpr (D != 2) {
+    if (all_j_equal(p->g, 6)) kern = k_interp<D, 6>;
+    if constexpr (D == 3) {
+      if (all_j_equal(p->g, 4)) kern = k_interp<D, 4>;
+      if (all_j_equal(p->g, 5)) kern = k_interp<D, 5>;
+      if (all_j_equal(p->g, 7)) kern = k_interp<D, 7>;
+    }
+  }
   kern<<<gd, 256, 0, p->stream>>>(grid, y, P, p->g, p->Kprod, p->M);
   return cudaGetLastError();
 }

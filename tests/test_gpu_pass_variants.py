@@ -102,6 +102,20 @@ def test_3d_interpolation_and_gridding(nf, J, Kd, M):
         assert rel(plan.gridding(dev(y)).cpu().numpy(), oracle.gridding_VH(p, y)) < TOL_V
 
 
+# 3D interpolation on both sides of the CTA rule, one transform and a batch
+@pytest.mark.parametrize("J", [4, 5, 6, 7])
+@pytest.mark.parametrize("K,M,nb", [(48, 9000, 1), (128, 9000, 1), (64, 4001, 3), (64, 4001, 17)])
+def test_3d_chunk_and_point_kernels(nf, J, K, M, nb):
+    om = W.uniform_random_om(M, 3, seed=15)
+    Kd, Nd = (K,) * 3, (K // 4 * 2, K // 4 * 2, K // 4 * 2)
+    p = oracle.make_plan(om, Nd, Kd, (J,) * 3)
+    xs = cn((nb,) + Nd, 16)
+    with nf.NufftPlan(dev(om), Nd, Kd, (J,) * 3) as plan:
+        yb = plan.forward_batch(dev(xs)).cpu().numpy()
+    for b in {0, nb - 1}:
+        assert rel(yb[b], oracle.forward(p, xs[b])) < TOL_OP
+
+
 # 2D single transforms: tiles of 16 and others, chunk counts at the edges of a chunk
 @pytest.mark.parametrize("Jd", [(4, 4), (5, 5), (6, 6), (7, 7), (7, 4), (1, 6)])
 @pytest.mark.parametrize("Kd,M", [((64, 48), 255), ((32, 32), 1025), ((36, 90), 4100), ((18, 64), 40)])
