@@ -480,9 +480,9 @@ cudaError_t launch_LE(const FftArgs& A, int nb, cudaStream_t st, int64_t* nblock
 
 // Sixteen values per thread on strided axes of 128 to 512 points that still fill
 // the GPU: one hand-off instead of two for 128 and 256 points, fewer twiddles per
-// value, and 128-byte rows (64-byte ones for 512) (on a 256^3 grid's passes
-// 30 -> 24 us and 54 -> 40 us forward; 8 frames of 32 512^2 coil images 1681 ->
-// 1652 us).  The contiguous passes lose more to the registers and the scaling's
+// value, and 128-byte rows, 64-byte ones for 512 (with the hand-offs above, a
+// 256^3 grid's transform 105 -> 81 us forward, 104 -> 69 us inverse, L2 flushed;
+// 8 frames of 32 512^2 coil images 1681 -> 1652 us).  The contiguous passes lose more to the registers and the scaling's
 // loads (those frames 1874 us), and a small pass is bound by latency: both take
 // eight, with twice the warps.
 constexpr int64_t kWideWarps = 8 * 152;

@@ -285,6 +285,8 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
 // registers a round ahead; the axis-0 and axis-1 ones reach the point's other
 // lanes through a per-warp strip of shared memory.  The J axis-1 taps of a row
 // are taken two at a time (fma2 on the pairs (re_j, re_j+1) and (im_j, im_j+1)).
+// 128^3 kooshball: 338 us with sub-batches between barriers, 271 us so; bound by
+// the shared-memory pipe (86 % busy): two loads per tap.
 template <int JF>
 struct Chunk3dCfg {
   static constexpr int kThreads = 512;
@@ -799,7 +801,8 @@ __device__ __forceinline__ void scatter_chunk(int* acc, const int ncell, const f
 // of a point loads the l-th coefficient of each axis into registers a round
 // ahead, and the axis-0 and axis-1 ones are passed to the point's other lanes
 // through a per-warp strip of shared memory.  A chunk that needs three words
-// takes scatter_chunk.
+// takes scatter_chunk.  128^3 kooshball: 517 us with three words throughout, 324 us
+// so, with the shared-memory pipe 78 % and the issue slots 66 % busy.
 // rn(x) as an integer for |x| < 1.2e9 on the FP32 and integer pipes: three
 // additions and a shift-add, against one F2I, which the conversion unit issues
 // at one warp per two cycles and SM.  t holds x rounded to a multiple of 512
@@ -1428,7 +1431,7 @@ k_gridding_chunk2d(const float2* __restrict__ y_b, float2* __restrict__ tiles_b,
 // column, as k_gridding_reduce3d below does, so a 16^2 tile takes one warp and a
 // CTA several tiles.  The same sums in the same order as reduce_tile with one
 // group.  A frame of 32 coils on a 512^2 grid (32 x 1024 tiles): 55 us with 64
-// threads and a neighbour mask per cell.
+// threads and a neighbour mask per cell, 41 us so.
 constexpr int kRed2Rows = 8;
 constexpr int kRed2Threads = 256;
 
@@ -1480,7 +1483,8 @@ k_gridding_reduce2d(const float2* __restrict__ tiles_b, const int32_t* __restric
 // over the source bin's chunks, from zero, as in reduce_tile (the same values).
 // CTA x: tile x / nsl, slice x % nsl = (column block, z0).  Measured on the
 // 128^3 kooshball (4096 tiles of 16^3, 226 MB of partial tiles, 134 MB of grid):
-// 184 us with four cells per thread and a neighbour mask for each.
+// 184 us with four cells per thread and a neighbour mask for each, 112 us so with
+// three CTAs per SM; four take another 10 us off.
 constexpr int kRed3Planes = 8;
 constexpr int kRed3Threads = 256;
 
