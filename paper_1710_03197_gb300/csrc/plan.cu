@@ -751,12 +751,33 @@ int validate_om(nufft_plan_t* p, const float* om) {
   return NUFFT_OK;
 }
 
+// Host lists of build_points: tile starts from the device, and the chunk list,
+// the chunk ranges and the 2D work list to it.  A copy from pageable memory may
+// read its source at any time up to a wait (a host whose pages the GPU can read
+// in place need not stage it), so the caller holds the lists until the wait that
+// ends its call, and clears `pending` after it; on any other way out the
+// destructor waits before the lists go.
+struct HostLists {
+  cudaStream_t stream;
+  bool pending = true;
+  std::vector<int32_t> bin_start, bin_chunk;
+  std::vector<Chunk> chunks;
+  std::vector<int4> work;
+  explicit HostLists(cudaStream_t st) : stream(st) {}
+  HostLists(const HostLists&) = delete;
+  HostLists& operator=(const HostLists&) = delete;
+  ~HostLists() {
+    if (pending) cudaStreamSynchronize(stream);
+  }
+};
+
 // Everything that depends on the trajectory (validated already): the tile
 // sort, the chunk list (chunks and partial tiles grown when it needs more),
 // the bank order, the per-point interpolator and, once the trajectory
 // gradient has been used, its derivative.  The per-dimension tables, the
-// Chebyshev expansions and every other buffer are the plan's already.
-int build_points(nufft_plan_t* p, const float* om) {
+// Chebyshev expansions and every other buffer are the plan's already.  Copies
+// out of `lists` may still be in flight on return.
+int build_points(nufft_plan_t* p, const float* om, HostLists& lists) {
   Geom& g = p->g;
   const int d = g.d;
   const int64_t M = p->M;
@@ -791,12 +812,14 @@ int build_points(nufft_plan_t* p, const float* om) {
   }
 
   // ---- gridding work list: each tile's points cut into chunks
-  std::vector<int32_t> bs(g.nbins + 1);
+  std::vector<int32_t>& bs = lists.bin_start;
+  bs.resize(g.nbins + 1);
   NUFFT_CUDA_TRY(p, cudaMemcpyAsync(bs.data(), p->bin_start, (g.nbins + 1) * sizeof(int32_t), cudaMemcpyDeviceToHost,
                                     st));
   NUFFT_CUDA_TRY(p, cudaStreamSynchronize(st));
-  std::vector<Chunk> ch;
-  std::vector<int32_t> bc(g.nbins + 1);
+  std::vector<Chunk>& ch = lists.chunks;
+  std::vector<int32_t>& bc = lists.bin_chunk;
+  bc.resize(g.nbins + 1);
   for (int64_t b = 0; b < g.nbins; ++b) {
     bc[b] = (int32_t)ch.size();
     for (int32_t s0 = bs[b]; s0 < bs[b + 1]; s0 += kChunkPoints[d]) {
@@ -859,7 +882,7 @@ int build_points(nufft_plan_t* p, const float* om) {
     reduce2d_groups(g.T[0] * g.T[1], &gsize, &ng);
     if (gsize * ng <= 256) {
       const int nb0 = g.nb[0], nb1 = g.nb[1];
-      std::vector<int4> wl;
+      std::vector<int4>& wl = lists.work;
       int pend[4] = {-1, -1, -1, -1}, fill = 0;
       for (int t = 0; t < (int)g.nbins; ++t) {
         const int b0 = t / nb1, b1 = t % nb1;
@@ -1007,13 +1030,15 @@ int build_plan(nufft_plan_t* p, const float* om) {
   NUFFT_CUDA_TRY(p, dalloc(p, &p->sort_vals, M));
   NUFFT_CUDA_TRY(p, dalloc(p, &p->sort_hist, M > 0 ? (int64_t)256 * sort_blocks(M) : 0));
   NUFFT_CUDA_TRY(p, dalloc(p, &p->perm2, M));
-  rc = build_points(p, om);
+  HostLists lists(st);
+  rc = build_points(p, om, lists);
   if (rc != NUFFT_OK) return rc;
   NUFFT_CUDA_TRY(p, dalloc(p, &p->grid, p->Kprod));
   NUFFT_CUDA_TRY(p, dalloc(p, &p->ytmp, M));
   NUFFT_CUDA_TRY(p, dalloc(p, &p->x_stage, p->Nprod));
   NUFFT_CUDA_TRY(p, dalloc(p, &p->y_stage, M));
   NUFFT_CUDA_TRY(p, cudaStreamSynchronize(st));
+  lists.pending = false;
   return NUFFT_OK;
 }
 
@@ -1247,9 +1272,11 @@ extern "C" int nufft_plan_set_trajectory(nufft_plan_t* p, const float* om_dev) {
     release_toeplitz(p);
     p->normal_op = 0;
   }
-  rc = build_points(p, om_dev);
+  HostLists lists(p->stream);
+  rc = build_points(p, om_dev, lists);
   if (rc != NUFFT_OK) return rc;
   NUFFT_CUDA_TRY(p, cudaStreamSynchronize(p->stream));
+  lists.pending = false;
   return NUFFT_OK;
 }
 
