@@ -344,13 +344,15 @@ __device__ void minmax_coefs(double theta1, int N, int K, int J, const double* s
 // expansion is checked against the sums at other points of [0, 1] and used
 // only where it agrees to kChebTol relative to the largest coefficient.
 //
-// The expansions fall off fast (J = 4 to 9: below 1e-12 of the largest from the
-// 13th term), so the first kMono terms are also kept as a polynomial in x: one
-// multiply-add per term and component instead of the recurrence's two FP64
-// operations over all 24 (32,768 points in 2D: 85 us, FP64-bound).  It is checked
-// against the sums the same way and used where it agrees to the same tolerance.
+// The expansions fall off fast, so the first kMono terms are also kept as a
+// polynomial in x: one multiply-add per term and component instead of the
+// recurrence's two FP64 operations over all 24 (32,768 points in 2D: 85 us,
+// FP64-bound).  With 16 terms what is left out is below the rounding of the
+// evaluation for every N / K (14 terms left up to 8e-14 of the largest derivative
+// where N = K, twenty times the expansion's error).  It is checked against the
+// sums the same way and used where it agrees to the same tolerance.
 constexpr int kCheb = 24;
-constexpr int kMono = 14;
+constexpr int kMono = 16;
 constexpr double kChebTol = 1e-10;
 
 __device__ __forceinline__ double cheb_node(int m) { return cos(kPi * (m + 0.5) / kCheb); }
