@@ -495,24 +495,25 @@ cudaError_t launch_LE(const FftArgs& A, int nb, cudaStream_t st, int64_t* nblock
   if constexpr (!STRIDED) {
     if (A.pro_p || A.epi_part) return go(k_fft_pass<L, E, STRIDED, INV, true, 0>);
   } else {
-    constexpr int kFull = E == 16 ? (L == 512 ? 3 : 4) : 3;
+    constexpr int kFull = E == 16 ? 4 : 3;
     if (wlog == kFull) return go(k_fft_pass<L, E, STRIDED, INV, false, kFull>);
   }
   return go(k_fft_pass<L, E, STRIDED, INV, false, 0>);
 }
 
-// Sixteen values per thread on strided axes of 128 to 512 points that still fill
-// the GPU: one hand-off instead of two for 128 and 256 points, fewer twiddles per
-// value, and 128-byte rows, 64-byte ones for 512 (with the hand-offs above, a
-// 256^3 grid's transform 105 -> 81 us forward, 104 -> 69 us inverse, L2 flushed;
-// 8 frames of 32 512^2 coil images 1681 -> 1652 us).  The contiguous passes lose more to the registers and the scaling's
-// loads (those frames 1874 us), and a small pass is bound by latency: both take
-// eight, with twice the warps.
+// Sixteen values per thread on strided axes of 128 and 256 points that still fill
+// the GPU: one hand-off instead of two, fewer twiddles per value, and 128-byte rows
+// (with the hand-offs above, a 256^3 grid's transform 105 -> 81 us forward, 104 ->
+// 69 us inverse, L2 flushed; the error against 64 bits falls by a fifth).  Lines of
+// 512 points need two hand-offs either way: 2 % faster with sixteen values on 32
+// coils of 512^2, but a smooth image's samples are 1.22 times further off.  The
+// contiguous passes lose more to the registers and the scaling's loads, and a small
+// pass is bound by latency: all these take eight, with twice the warps.
 constexpr int64_t kWideWarps = 8 * 152;
 
 template <int L, bool STRIDED, bool INV>
 cudaError_t launch_L(const FftArgs& A, int nb, cudaStream_t st, int64_t* nblocks, bool query) {
-  if constexpr (STRIDED && (L == 128 || L == 256 || L == 512)) {
+  if constexpr (STRIDED && (L == 128 || L == 256)) {
     if (A.nouter * A.inner * nb * (L / 16) >= kWideWarps * 32 && A.inner % 16 == 0)
       return launch_LE<L, 16, STRIDED, INV>(A, nb, st, nblocks, query);
   }
