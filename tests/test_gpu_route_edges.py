@@ -1,0 +1,56 @@
+"""Kernels behind a rule on sizes, at the sizes where a rule changes its mind.
+
+Tolerances as for the pass variants: an FFT line of 1024 points has 10 radix-2 levels of at
+most about 1.5 * 2^-24 in the 2-norm, two axes 1.8e-6 if all errors added up: 2e-6;
+interpolation and gridding about eight roundings of 2^-24 per contribution: 1e-6.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL_FFT = 2e-6
+TOL_V = 1e-6
+TOL_OP = TOL_FFT + TOL_V
+
+
+@pytest.fixture(scope="module")
+def nf():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1710_03197_gb300 as nf
+    return nf
+
+
+def rel(a, b):
+    return float(np.linalg.norm(np.ravel(a) - np.ravel(b)) / np.linalg.norm(b))
+
+
+def cn(shape, seed):
+    rng = np.random.default_rng(seed)
+    return (rng.standard_normal(shape) + 1j * rng.standard_normal(shape)).astype(np.complex64)
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+# strided lines that are no powers of two with CTAs enough for 4 to 16 columns: threads
+# that take one butterfly of the smallest radix, and threads that take several
+@pytest.mark.parametrize("L,other,nb", [(54, 288, 17), (250, 288, 9), (360, 288, 9), (384, 96, 26), (500, 144, 17),
+                                        (750, 96, 13), (1000, 96, 13), (972, 36, 34)])
+def test_mixed_radix_columns_of_a_batch(nf, L, other, nb):
+    Kd = (L, other)
+    Nd = tuple(2 * max(1, K // 3) for K in Kd)
+    om = W.uniform_random_om(701, 2, seed=L)
+    p = oracle.make_plan(om, Nd, Kd, (4, 4))
+    xs, ys = cn((nb,) + Nd, 1), cn((nb, om.shape[0]), 2)
+    with nf.NufftPlan(dev(om), Nd, Kd, (4, 4)) as plan:
+        yb, xb = plan.forward_batch(dev(xs)).cpu().numpy(), plan.adjoint_batch(dev(ys)).cpu().numpy()
+    for b in {0, nb - 1}:
+        assert rel(yb[b], oracle.forward(p, xs[b])) < TOL_OP
+        assert rel(xb[b], oracle.adjoint(p, ys[b])) < TOL_OP
