@@ -449,10 +449,10 @@ k_interp_chunk3d(const float2* __restrict__ grid_b, float2* __restrict__ y_b, co
 // one thread per point (first neighbours, the J0 + J1 coefficients, permutation
 // or sample), so a CTA waits for one round of global loads instead of one per
 // pass of its warps over the chunk.  Layout: c0[J0][cap] (row by row: the lanes
-// of a point read one value), c1[cap][J1 | 1] (point by point: the lanes of a
-// point read consecutive words; the odd pitch keeps the staging threads' stores
-// on distinct banks, 2- to 4-way conflicts otherwise), k[2][cap] (first neighbours
-// relative to the tile origin).
+// of a point read one value), c1[cap][pitch1] (point by point: the lanes of a
+// point read consecutive words; an odd pitch keeps the staging threads' stores
+// on distinct banks, 2- to 4-way conflicts otherwise, see staged_pitch), k[2][cap]
+// (first neighbours relative to the tile origin).
 // JF > 0: J0 = J1 = JF; TF > 0: 16^2 tiles, so that the rows of a point's
 // neighbours are immediate offsets.
 struct Tile2d {
@@ -469,8 +469,20 @@ struct Staged2d {
   int* k;
   int pitch1;
   // float2 of shared memory per chunk for the coefficients
-  static size_t coefs(int J0, int J1) { return (size_t)kChunkPoints[2] * (J0 + (J1 | 1)); }
+  static size_t coefs(int J0, int pitch) { return (size_t)kChunkPoints[2] * (J0 + pitch); }
 };
+
+// pitch1 of the staged kernels: J1 | 1, or J1 where the odd pitch would cost a CTA per
+// SM (`rest` bytes of shared memory beside the coefficients).  J = 4 to 7 always have
+// room.  J = 16: three CTAs per SM, two with the odd pitch; 40,000 points on a
+// 360 x 288 grid (432 chunks) 17.7 us against 26.3.
+int staged_pitch(int J0, int J1, size_t rest) {
+  if (J0 == J1 && J0 >= 4 && J0 <= 7) return J1 | 1;   // fixed in the kernels
+  auto ctas = [&](int pitch) {   // 1 KB of each CTA's share is the system's
+    return (size_t)(228 * 1024) / (rest + Staged2d::coefs(J0, pitch) * sizeof(float2) + 1024);
+  };
+  return std::min<size_t>(4, ctas(J1 | 1)) < std::min<size_t>(4, ctas(J1)) ? J1 : J1 | 1;
+}
 
 template <int JF>
 __device__ __forceinline__ void stage_points2d(const Staged2d& S, const Points& P, const Geom& g, const Chunk& ch,
@@ -566,17 +578,17 @@ __device__ __forceinline__ void gather_staged2d(const Staged2d& S, const Chunk& 
 template <int JF, int TF>
 __global__ void __launch_bounds__(256, 4)
 k_interp_chunk2d(const float2* __restrict__ grid, float2* __restrict__ y, const Chunk* __restrict__ chunks,
-                 const Points P, const Geom g) {
+                 const Points P, const Geom g, const int pitch) {
   constexpr int cap = kChunkPoints[2];
   static_assert(cap == 256, "one thread per staged point");
   constexpr int PF = TF > 0 ? TF + JF - 1 : 0;
   extern __shared__ float tile[];
   const int ncell = PF > 0 ? PF * PF : (int)g.padded_cells;
-  const int J0 = JF > 0 ? JF : g.J[0], J1 = JF > 0 ? JF : g.J[1];
+  const int J0 = JF > 0 ? JF : g.J[0];
   Staged2d S;
   S.c0 = reinterpret_cast<float2*>(tile + 2 * ncell);   // 8-byte aligned: 2 * ncell floats
   S.c1 = S.c0 + J0 * cap;
-  S.pitch1 = J1 | 1;
+  S.pitch1 = JF > 0 ? JF | 1 : pitch;
   S.k = reinterpret_cast<int*>(S.c1 + S.pitch1 * cap);
   int* s_p = S.k + 2 * cap;
   const Chunk ch = chunks[blockIdx.x];
@@ -1253,7 +1265,8 @@ k_gridding_reduce_packed2d(const float2* __restrict__ tiles, const int32_t* __re
 template <int JF, int TF, bool FUSED>
 __global__ void __launch_bounds__(256, 4)
 k_gridding_chunk_staged(const float2* __restrict__ y_b, float2* __restrict__ tiles_b,
-                        const Chunk* __restrict__ chunks, const Points P, const Geom g, int64_t ybs, int64_t tbs) {
+                        const Chunk* __restrict__ chunks, const Points P, const Geom g, int64_t ybs, int64_t tbs,
+                        const int pitch) {
   constexpr int cap = kChunkPoints[2];
   static_assert(cap == 256, "one thread per staged point");
   constexpr int PF = TF > 0 ? TF + JF - 1 : 0;
@@ -1267,7 +1280,7 @@ k_gridding_chunk_staged(const float2* __restrict__ y_b, float2* __restrict__ til
   Staged2d S;
   S.c0 = reinterpret_cast<float2*>(acc + 2 * ncell);   // 8-byte aligned: 2 * ncell words
   S.c1 = S.c0 + J0 * cap;
-  S.pitch1 = J1 | 1;
+  S.pitch1 = JF > 0 ? JF | 1 : pitch;
   float2* s_y = S.c1 + S.pitch1 * cap;
   S.k = reinterpret_cast<int*>(s_y + cap);
   const Chunk ch = chunks[blockIdx.x];
@@ -1628,12 +1641,13 @@ cudaError_t interp_chunks(const nufft_plan_t* p, const float2* grid, float2* y, 
   for (int a = 0; a < D; ++a) t16 = t16 && p->g.T[a] == 16;
   if constexpr (D == 2) {
     const int J0 = p->g.J[0], J1 = p->g.J[1];
-    const size_t smem = (size_t)p->g.padded_cells * 2 * sizeof(float) + Staged2d::coefs(J0, J1) * sizeof(float2) +
-                        (size_t)kChunkPoints[2] * 3 * sizeof(int);
+    const size_t rest = (size_t)p->g.padded_cells * 2 * sizeof(float) + (size_t)kChunkPoints[2] * 3 * sizeof(int);
+    const int pitch = staged_pitch(J0, J1, rest);
+    const size_t smem = rest + Staged2d::coefs(J0, pitch) * sizeof(float2);
     auto go = [&](auto kern) {
       cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
-      kern<<<(unsigned)p->nchunks, kChunkPoints[2], smem, p->stream>>>(grid, y, p->chunks, P, p->g);
+      kern<<<(unsigned)p->nchunks, kChunkPoints[2], smem, p->stream>>>(grid, y, p->chunks, P, p->g, pitch);
       return cudaGetLastError();
     };
     switch (J0 == J1 ? J0 : 0) {
@@ -1774,14 +1788,15 @@ cudaError_t launch_chunks(const nufft_plan_t* p, const float2* y, float2* tiles,
   if constexpr (D == 2) {
     const int J0 = p->g.J[0], J1 = p->g.J[1];
     const bool t16 = p->g.T[0] == 16 && p->g.T[1] == 16;
-    const size_t smem = (size_t)p->g.padded_cells * Fix<2>::kWords * sizeof(int) +
-                        (Staged2d::coefs(J0, J1) + kChunkPoints[2]) * sizeof(float2) +
-                        (size_t)kChunkPoints[2] * 2 * sizeof(int) +
+    const size_t rest = (size_t)p->g.padded_cells * Fix<2>::kWords * sizeof(int) +
+                        (size_t)kChunkPoints[2] * (sizeof(float2) + 2 * sizeof(int)) +
                         (FUSED ? (size_t)p->g.padded_cells * 2 * sizeof(float) : 0);
+    const int pitch = staged_pitch(J0, J1, rest);
+    const size_t smem = rest + Staged2d::coefs(J0, pitch) * sizeof(float2);
     auto go = [&](auto kern) {
       e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
-      kern<<<gd, kChunkPoints[2], smem, p->stream>>>(y, tiles, p->chunks, P, p->g, ybs, tbs);
+      kern<<<gd, kChunkPoints[2], smem, p->stream>>>(y, tiles, p->chunks, P, p->g, ybs, tbs, pitch);
       return cudaGetLastError();
     };
     switch (J0 == J1 ? J0 : 0) {

@@ -54,3 +54,16 @@ def test_mixed_radix_columns_of_a_batch(nf, L, other, nb):
     for b in {0, nb - 1}:
         assert rel(yb[b], oracle.forward(p, xs[b])) < TOL_OP
         assert rel(xb[b], oracle.adjoint(p, ys[b])) < TOL_OP
+
+
+# staged 2D kernels whose coefficients lose the odd pitch for a third CTA per SM, and keep it
+@pytest.mark.parametrize("Jd", [(16, 16), (16, 14), (13, 16), (15, 15)])
+@pytest.mark.parametrize("Kd", [(360, 288), (64, 80)])
+def test_2d_many_neighbours(nf, Jd, Kd):
+    Nd = tuple(K // 10 * 8 for K in Kd)   # a lean grid: G is well conditioned
+    om = W.uniform_random_om(1500, 2, seed=5)
+    p = oracle.make_plan(om, Nd, Kd, Jd)
+    z, y = cn(Kd, 5), cn(1500, 6)
+    with nf.NufftPlan(dev(om), Nd, Kd, Jd) as plan:
+        assert rel(plan.interp(dev(z)).cpu().numpy(), oracle.interp_V(p, z)) < TOL_V
+        assert rel(plan.gridding(dev(y)).cpu().numpy(), oracle.gridding_VH(p, y)) < TOL_V
