@@ -1284,6 +1284,14 @@ k_gridding_chunk_staged(const float2* __restrict__ y_b, float2* __restrict__ til
   float2* s_y = S.c1 + S.pitch1 * cap;
   S.k = reinterpret_cast<int*>(s_y + cap);
   const Chunk ch = chunks[blockIdx.x];
+  // Loops over the cells take their number from the plan even where it is a constant:
+  // unrolled they cost the chunks of a few points more than they save (1024^2 grid,
+  // 40,000 points 14.5 us, 12.8 so; 512^2, 200,000 points 10.5, 10.0).
+  const int cells = (int)g.padded_cells;
+  auto zero = [&] {
+    for (int c = threadIdx.x; c < cells; c += blockDim.x) reinterpret_cast<int2*>(acc)[c] = make_int2(0, 0);
+  };
+  if (!FUSED) zero();   // while the chunk's entry is on its way
   const Tile2d T = tile_origin2d(g, ch.bin);
   const int qs = threadIdx.x;   // the point this thread stages
   int pm = 0;
@@ -1292,8 +1300,8 @@ k_gridding_chunk_staged(const float2* __restrict__ y_b, float2* __restrict__ til
   if (FUSED) {
     float* gre = reinterpret_cast<float*>(S.k + 2 * cap);   // the chunk's padded tile of the spectrum
     stage_tile2d<PF>(y, g, T, gre, gre + ncell);
+    zero();
   }
-  for (int c = threadIdx.x; c < ncell; c += blockDim.x) reinterpret_cast<int2*>(acc)[c] = make_int2(0, 0);
   if (!FUSED && qs < ch.count) s_y[qs] = __ldg(&y[pm]);
   __syncthreads();
   if (FUSED) {
@@ -1324,7 +1332,7 @@ k_gridding_chunk_staged(const float2* __restrict__ y_b, float2* __restrict__ til
   }
   __syncthreads();
   float2* out = tiles + (int64_t)ch.slot * g.padded_cells;
-  for (int c = threadIdx.x; c < ncell; c += blockDim.x) out[c] = fix_value<2>(acc, ncell, c, cs);
+  for (int c = threadIdx.x; c < cells; c += blockDim.x) out[c] = fix_value<2>(acc, ncell, c, cs);
 }
 
 // ---------------------------------------------------------------- 2D chunk passes of a batch
