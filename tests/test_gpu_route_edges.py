@@ -56,6 +56,20 @@ def test_mixed_radix_columns_of_a_batch(nf, L, other, nb):
         assert rel(xb[b], oracle.adjoint(p, ys[b])) < TOL_OP
 
 
+# V of a 2D batch: CTAs below and above the number from which a thread takes four elements
+@pytest.mark.parametrize("J,M,nb", [(4, 41000, 16), (4, 41000, 17), (5, 30000, 17), (6, 25000, 13), (6, 25000, 12),
+                                    (7, 17000, 18), (7, 700, 5)])
+def test_2d_batch_interpolation(nf, J, M, nb):
+    Kd, Nd = (90, 80), (54, 48)
+    om = W.uniform_random_om(M, 2, seed=J)
+    p = oracle.make_plan(om, Nd, Kd, (J, J))
+    xs = cn((nb,) + Nd, 3)
+    with nf.NufftPlan(dev(om), Nd, Kd, (J, J)) as plan:
+        yb = plan.forward_batch(dev(xs)).cpu().numpy()
+    for b in {0, 3, 4, nb - 1}:
+        assert rel(yb[b], oracle.forward(p, xs[b])) < TOL_OP
+
+
 # staged 2D kernels whose coefficients lose the odd pitch for a third CTA per SM, and keep it
 @pytest.mark.parametrize("Jd", [(16, 16), (16, 14), (13, 16), (15, 15)])
 @pytest.mark.parametrize("Kd", [(360, 288), (64, 80)])
