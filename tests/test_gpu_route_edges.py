@@ -81,3 +81,19 @@ def test_2d_many_neighbours(nf, Jd, Kd):
     with nf.NufftPlan(dev(om), Nd, Kd, Jd) as plan:
         assert rel(plan.interp(dev(z)).cpu().numpy(), oracle.interp_V(p, z)) < TOL_V
         assert rel(plan.gridding(dev(y)).cpu().numpy(), oracle.gridding_VH(p, y)) < TOL_V
+
+
+# 1D: one tile's list of 1 to 40 chunks over four thread groups, three pairs in flight.  A
+# chunk's sums round by up to 2^-31 B per contribution, B < 2 max|c| sum(|Re y| + |Im y|) over its
+# points; a wrong list is off by whole contributions.
+@pytest.mark.parametrize("K,M", [(64, 300), (64, 1025), (500, 2049), (1000, 5000), (64, 7000), (1024, 9001), (96, 40001)])
+def test_1d_reduction(nf, K, M):
+    om = W.uniform_random_om(M, 1, seed=M)
+    p = oracle.make_plan(om, (K // 2,), (K,), (6,))
+    y = cn(M, 8)
+    with nf.NufftPlan(dev(om), (K // 2,), (K,), (6,)) as plan:
+        got = plan.gridding(dev(y)).cpu().numpy()
+    ref = oracle.gridding_VH(p, y)
+    sums = (np.abs(y.real) + np.abs(y.imag)).sum()
+    fixed = min(M, 1024) * 2.0 ** -31 * 2 * np.abs(p.coef[0]).max() * sums
+    assert np.abs(got - ref).max() <= fixed + TOL_V * np.linalg.norm(ref)
