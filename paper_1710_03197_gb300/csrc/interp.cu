@@ -1545,9 +1545,18 @@ k_gridding_reduce2d(const float2* __restrict__ tiles_b, const int32_t* __restric
 // 128^3 kooshball (4096 tiles of 16^3, 226 MB of partial tiles, 134 MB of grid):
 // 184 us with four cells per thread and a neighbour mask for each, 112 us so with
 // three CTAs per SM; four take another 10 us off.
-constexpr int kRed3Planes = 8;
+// kPlanes = 8, one pair in flight, for tiles of few (neighbour, chunk) pairs.  A tile
+// of many pairs is one chain: kPlanes = 2 gives it four times the CTAs, kDepth = 4 as
+// many loads in flight, and a pair of the chain 0.11 us instead of 0.33; but each
+// cell's share of the set-up grows, 0.05 us per 4096 cells of grid instead of 0.02.
+// So the longest list, max_pairs, decides against the grid's size (kDensePairs).
+// 8 / 2 planes: 300,000 clustered points on 64^3 (152 pairs) 51 / 19 us, kooshballs
+// 128^3 with 1,000,000 points (153) 55 / 41, 128^3 with 307,200 (48) 21 / 30, 64^3
+// with 100,000 (33) 12.8 / 8.2, eight of these 21 / 32.
 constexpr int kRed3Threads = 256;
+constexpr int64_t kDensePairs = 24000;   // grid cells (times batch elements) per pair
 
+template <int kRed3Planes, int kDepth>
 __global__ void __launch_bounds__(kRed3Threads, 4)
 k_gridding_reduce3d(const float2* __restrict__ tiles_b, const int32_t* __restrict__ bin_chunk,
                     float2* __restrict__ grid_b, const Geom g, int64_t tbs, int64_t gbs, int nsl, int nz) {
@@ -1578,6 +1587,21 @@ k_gridding_reduce3d(const float2* __restrict__ tiles_b, const int32_t* __restric
     int q = __ldg(&bin_chunk[src]);
     const float2* ptr = tiles + (int64_t)q * g.padded_cells +
                         ((z0 + e0 * g.T[0]) * g.P[1] + r1 + e1 * g.T[1]) * g.P[2] + r2 + e2 * g.T[2];
+    if constexpr (kDepth > 1) {
+      for (; q + kDepth <= q1; q += kDepth, ptr += kDepth * g.padded_cells) {
+        float2 v[kDepth][kRed3Planes];
+#pragma unroll
+        for (int u = 0; u < kDepth; ++u)
+#pragma unroll
+          for (int k = 0; k < kRed3Planes; ++k)
+            v[u][k] = k < n ? __ldg(&ptr[u * g.padded_cells + k * plane]) : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < kDepth; ++u)
+#pragma unroll
+          for (int k = 0; k < kRed3Planes; ++k)
+            if (k < n) acc[k] = cadd(acc[k], v[u][k]);
+      }
+    }
     if (n == kRed3Planes) {
       for (; q < q1; ++q, ptr += g.padded_cells) {
         float2 v[kRed3Planes];
@@ -1612,11 +1636,15 @@ cudaError_t launch_reduce(const nufft_plan_t* p, const float2* tiles, float2* gr
     const Geom& g = p->g;
     const int cols = g.T[1] * g.T[2];
     const int threads = std::min(kRed3Threads, (cols + 31) / 32 * 32);
-    const int nz = (g.T[0] + kRed3Planes - 1) / kRed3Planes;
-    const int nsl = nz * ((cols + threads - 1) / threads);
-    k_gridding_reduce3d<<<dim3((unsigned)(g.nbins * nsl), (unsigned)nb), threads, 0, p->stream>>>(
-        tiles, p->bin_chunk, grid, g, p->nchunks * g.padded_cells, p->Kprod, nsl, nz);
-    return cudaGetLastError();
+    auto go = [&](auto kern, int planes) {
+      const int nz = (g.T[0] + planes - 1) / planes;
+      const int nsl = nz * ((cols + threads - 1) / threads);
+      kern<<<dim3((unsigned)(g.nbins * nsl), (unsigned)nb), threads, 0, p->stream>>>(
+          tiles, p->bin_chunk, grid, g, p->nchunks * g.padded_cells, p->Kprod, nsl, nz);
+      return cudaGetLastError();
+    };
+    return p->max_pairs * kDensePairs > p->Kprod * nb ? go(k_gridding_reduce3d<2, 4>, 2)
+                                                      : go(k_gridding_reduce3d<8, 1>, 8);
   }
   if constexpr (D == 2) {
     if (nb > 1) {

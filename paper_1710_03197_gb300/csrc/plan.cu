@@ -753,6 +753,22 @@ int validate_om(nufft_plan_t* p, const float* om) {
   return NUFFT_OK;
 }
 
+// 3D: the most (neighbour, chunk) pairs that a tile's reduction sums: the chunks of
+// the tile and of its neighbours below, added up one axis at a time.
+int64_t longest_list3d(const Geom& g, const std::vector<int32_t>& bin_chunk) {
+  std::vector<int32_t> sum(g.nbins), prev(g.nbins);
+  for (int64_t b = 0; b < g.nbins; ++b) sum[b] = bin_chunk[b + 1] - bin_chunk[b];
+  int64_t stride = 1;
+  for (int a = 2; a >= 0; stride *= g.nb[a--]) {
+    prev = sum;
+    for (int64_t b = 0; b < g.nbins; ++b) {
+      const int64_t c = b / stride % g.nb[a];
+      sum[b] += prev[c > 0 ? b - stride : b + (g.nb[a] - 1) * stride];
+    }
+  }
+  return g.nbins > 0 ? *std::max_element(sum.begin(), sum.end()) : 0;
+}
+
 // Host lists of build_points: tile starts from the device, and the chunk list,
 // the chunk ranges and the 2D work list to it.  A copy from pageable memory may
 // read its source at any time up to a wait (a host whose pages the GPU can read
@@ -870,6 +886,7 @@ int build_points(nufft_plan_t* p, const float* om, HostLists& lists) {
     p->chunk_cap = nch;
   }
   p->nchunks = nch;
+  if (d == 3) p->max_pairs = longest_list3d(g, bc);
   if (nch > 0)
     NUFFT_CUDA_TRY(p, cudaMemcpyAsync(p->chunks, ch.data(), ch.size() * sizeof(Chunk), cudaMemcpyHostToDevice, st));
   NUFFT_CUDA_TRY(p, cudaMemcpyAsync(p->bin_chunk, bc.data(), bc.size() * sizeof(int32_t), cudaMemcpyHostToDevice,

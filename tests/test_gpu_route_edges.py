@@ -97,3 +97,21 @@ def test_1d_reduction(nf, K, M):
     sums = (np.abs(y.real) + np.abs(y.imag)).sum()
     fixed = min(M, 1024) * 2.0 ** -31 * 2 * np.abs(p.coef[0]).max() * sums
     assert np.abs(got - ref).max() <= fixed + TOL_V * np.linalg.norm(ref)
+
+
+# 3D tile sums: eight planes per thread, and two for lists of many chunks (1 to about 40 of
+# them), whole tiles and remainders of both, one transform and a batch
+@pytest.mark.parametrize("Kd,M,spread,nb", [((96, 96, 96), 9000, 3.1, 1), ((48, 48, 48), 9000, 3.1, 1),
+                                            ((48, 36, 50), 41000, 0.25, 1), ((32, 48, 32), 20000, 0.1, 1),
+                                            ((18, 20, 30), 9001, 3.1, 2), ((40, 64, 36), 21000, 0.3, 3)])
+@pytest.mark.parametrize("Jd", [(6, 6, 6), (3, 5, 4)])
+def test_3d_reduction(nf, Kd, M, spread, nb, Jd):
+    Nd = tuple(2 * (K // 4) for K in Kd)
+    om = (np.random.default_rng(M).uniform(-spread, spread, (M, 3))).astype(np.float32)
+    p = oracle.make_plan(om, Nd, Kd, Jd)
+    ys = cn((nb, M), 9)
+    with nf.NufftPlan(dev(om), Nd, Kd, Jd) as plan:
+        assert rel(plan.gridding(dev(ys[0])).cpu().numpy(), oracle.gridding_VH(p, ys[0])) < TOL_V
+        if nb > 1:
+            xb = plan.adjoint_batch(dev(ys)).cpu().numpy()
+            assert rel(xb[nb - 1], oracle.adjoint(p, ys[nb - 1])) < TOL_OP
