@@ -92,6 +92,7 @@ struct nufft_plan {
   nufft::Chunk* chunks;     // [nchunks]
   int32_t* bin_chunk;       // [nbins + 1] chunk range of each bin
   int64_t nchunks;
+  int longest_chunk;        // points of the longest chunk
   int64_t max_pairs;        // 3D: most (neighbour, chunk) pairs of a tile's reduction
   float2* tiles;            // [nchunks][padded_cells] gridding partial tiles
   float2* grid;             // [Kprod] oversampled grid work space

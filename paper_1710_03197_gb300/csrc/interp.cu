@@ -1741,26 +1741,44 @@ cudaError_t interp_chunks(const nufft_plan_t* p, const float2* grid, float2* y, 
   }
 }
 
-// 3D: CTAs from which the staged chunks beat the per-point kernel.  Measured, staged
-// against per point: 27 CTAs (9600 points) 43 us against 11, 200 (115,200) 46
-// against 32, 459 (307,200, with its gridding and FFTs) 176 against 217, 3044 (the
-// 128^3 pair) 855 against 1125; batches: 600 115 against 105, 1152 147 against
-// 148, 1600 234 against 267.
-constexpr int64_t kChunkCtas3d = 304, kChunkCtas3dBatch = 1024;
+// 3D, equal J from 4 to 7: whether the staged chunks beat the per-point kernel, from
+// estimates of both in us.  Staged: a set-up, then the longer of the longest chunk's
+// rounds (one CTA works them off alone) and all chunks' tiles and rounds over the SMs.
+// Per point: a floor that the chain of a point's loads takes, or all points' taps.
+// A round and a point cost in proportion to J^2 taps.  The constants are fitted to
+// 401 measurements of both (J = 4 to 7, grids 32^3 to 200^3, 300 to 1,000,000 random,
+// kooshball and clustered points, batches of 1 to 8; the staged ones within 20 % rms),
+// and the choice costs 3 % against the better of the two on average; a count of CTAs
+// alone cost 39 %.  Staged against per point, us: 64^3 grid, 300 points 5.9 / 7.7,
+// 10,000 kooshball points 37 / 8, 300,000 random points 48 / 66; 128^3, 300,000
+// clustered points 42 / 55 (151 chunks); 200^3, 100,000 random points 121 / 30
+// (8000 chunks); two of 100^3 with 100,000 kooshball points 73 / 45.  Batches overlap
+// their chunks less well than the estimate: they need a margin.
+bool staged_interp3d(const nufft_plan_t* p, int J, int nb) {
+  const double taps = J * J / 36.0;
+  const int per_warp = 32 / J, step = 16 * per_warp;   // points per round of a CTA
+  const double longest = (p->longest_chunk + step - 1) / step;
+  const double rounds = (double)p->M / step + 0.5 * p->nchunks;   // of all chunks
+  const double tile = 0.6 + 1.8 * (double)p->g.padded_cells / 9261;
+  const double staged = 4.0 + 1.4 * taps +
+                        std::max(1.5 * taps * longest, nb * (p->nchunks * tile + 1.7 * taps * rounds) / 152);
+  const double point = std::max(2.0 + 6.0 * taps, 1.2e-3 * taps * (double)p->M * nb / per_warp);
+  return staged * (nb > 1 ? 1.8 : 1.0) < point;
+}
 
 template <int D>
 cudaError_t interp_d(const nufft_plan_t* p, const float2* grid, float2* y, int nb) {
   // 2D: single transforms gather from staged tiles, batches per point (the chunk
   // kernel would stage each chunk's point data once per batch element: the
   // 32-coil frames' normal operator 2.36 -> 2.87 ms).
-  // 3D: staged tiles where the chunks (times batch elements) give the GPU CTAs
-  // enough; fewer are bound by the longest chunk's rounds.
+  // 3D: staged tiles where staged_interp3d expects them to win; J that it does not
+  // cover, single transforms.
   if constexpr (D == 2) {
     if (nb == 1) return interp_chunks<D>(p, grid, y, nb);
   }
   if constexpr (D == 3) {
     const int J = all_j_equal(p->g, p->g.J[0]) ? p->g.J[0] : 0;
-    if (J >= 4 && J <= 7 ? p->nchunks * nb >= (nb == 1 ? kChunkCtas3d : kChunkCtas3dBatch) : nb == 1)
+    if (J >= 4 && J <= 7 ? staged_interp3d(p, J, nb) : nb == 1)
       return interp_chunks<D>(p, grid, y, nb);
   }
   const Points P = points_view(p);

@@ -864,6 +864,7 @@ int build_points(nufft_plan_t* p, const float* om, HostLists& lists) {
     std::vector<Chunk> sorted(ch.size());
     for (const Chunk& c : ch) sorted[pos[most - c.count]++] = c;
     ch.swap(sorted);
+    p->longest_chunk = ch.empty() ? 0 : ch[0].count;
   }
   if (nch > p->chunk_cap) {   // grow the chunk list and the partial tiles (and the batched ones, lazily)
     drop_graphs(p);

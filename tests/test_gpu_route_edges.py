@@ -115,3 +115,61 @@ def test_3d_reduction(nf, Kd, M, spread, nb, Jd):
         if nb > 1:
             xb = plan.adjoint_batch(dev(ys)).cpu().numpy()
             assert rel(xb[nb - 1], oracle.adjoint(p, ys[nb - 1])) < TOL_OP
+
+
+def _kernels(f):
+    """Names of the kernels that f launches, empty where the profiler sees none."""
+    from torch.profiler import ProfilerActivity, profile
+    f()
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        f()
+        torch.cuda.synchronize()
+    return " ".join(e.key for e in prof.key_averages())
+
+
+def _first(J):
+    """Lowest frequency, in grid cells, whose first neighbour is cell 0."""
+    return (J - 1) // 2 - 0.5 * (J % 2)
+
+
+def _tile(om, K, J, T):
+    """Tile of each point's first neighbour on a K^3 grid."""
+    t = np.zeros(om.shape[0], dtype=np.int64)
+    for a in range(3):
+        t = t * (K // T) + (oracle.offsets_1d(om[:, a].astype(np.float64), K, J).astype(np.int64) + 1) % K // T
+    return t
+
+
+# 3D V by staged chunks on tiles of 10, with chunks of one round of the CTA's warps, one point
+# more, several rounds and the longest there is; and by points
+@pytest.mark.parametrize("J,M,staged", [(4, 1000000, True), (5, 600000, True), (6, 300000, True), (7, 300000, True),
+                                        (6, 300, False), (7, 9000, False), (4, 30000, False)])
+def test_3d_interpolation_routes(nf, J, M, staged):
+    K, N, T = 100, 50, 10
+    rng = np.random.default_rng(J)
+    om = rng.uniform(-np.pi, np.pi, (M, 3)).astype(np.float32)
+    step = 16 * (32 // J)
+    picks = []
+    if M >= 300000:   # tiles that hold exactly these numbers of points
+        sizes = {0: step, 111: step + 1, 222: 3 * step + 5, 333: 1, 444: 2048, 555: 2049}
+        om = om[~np.isin(_tile(om, K, J, T), list(sizes))]
+        for t, n in sizes.items():
+            corner = np.array([t // 100, t // 10 % 10, t % 10]) * T
+            u = corner + _first(J) + rng.uniform(0.1, T - 0.1, (n, 3))
+            w = (2 * np.pi / K * (u - K * (u > K / 2))).astype(np.float32)
+            w = w[_tile(w, K, J, T) == t]
+            assert w.shape[0] == n
+            picks.append(np.arange(om.shape[0], om.shape[0] + n))
+            om = np.concatenate([om, w])
+    picks = np.concatenate(picks + [rng.integers(0, om.shape[0], 1000)])
+    z = cn((K,) * 3, 10)
+    p = oracle.make_plan(om[picks], (N,) * 3, (K,) * 3, (J,) * 3)
+    with nf.NufftPlan(dev(om), (N,) * 3, (K,) * 3, (J,) * 3) as plan:
+        zd = dev(z)
+        got = plan.interp(zd).cpu().numpy()
+        plan.set_graphs(False)
+        names = _kernels(lambda: plan.interp(zd))
+    assert rel(got[picks], oracle.interp_V(p, z)) < TOL_V
+    if "k_interp" in names:
+        assert ("k_interp_chunk3d" in names) == staged, names
