@@ -525,11 +525,18 @@ __global__ void k_coef_max(const float2* coef, int64_t M, int d, int J0, int J1,
 // points of at most 2^20 + 1: no overflow), so W does not depend on the order
 // of the atomics.  Lane layout and bank order are the gridding's; one atomic
 // and no samples, so about a third of its time.
-// JF > 0: every J is JF, the axis-1 magnitudes sit in registers.  A weight w < 2^21
-// is rounded up by adding 2^23 towards +infinity: the low mantissa bits are the
+// JF > 0: every J is JF, the magnitudes of axes 0 and 1 sit in registers; JF = 0: in a
+// strip of shared memory per warp, after the cells (taken from global memory again for
+// every tap they made the pass for J = 9, 100,000 points, 454 us long, 135 so).  A weight
+// w < 2^21 is rounded up by adding 2^23 towards +infinity: the low mantissa bits are the
 // integer, no conversion instruction.
+constexpr int kWmaxThreads = 512;
+size_t wmax_smem(const Geom& g, bool fixed) {
+  const size_t strip = fixed ? 0 : (size_t)(kWmaxThreads / 32) * (g.J[0] + g.J[1]) * (32 / g.J[2]);
+  return ((size_t)g.padded_cells + strip) * sizeof(uint32_t);
+}
 template <int JF>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(kWmaxThreads)
 k_chunk_wmax(Chunk* chunks, const int32_t* kf, const float2* coef, int64_t off1, int64_t off2, int64_t M, const Geom g,
              const uint32_t* cmax) {
   extern __shared__ uint32_t wacc[];
@@ -553,28 +560,44 @@ k_chunk_wmax(Chunk* chunks, const int32_t* kf, const float2* coef, int64_t off1,
   auto mag = [](float2 c) { return sqrtf(c.x * c.x + c.y * c.y); };
   const int G = JF > 0 ? JF : g.J[2], J0 = JF > 0 ? JF : g.J[0], J1 = JF > 0 ? JF : g.J[1];
   const int lane = threadIdx.x & 31, per_warp = 32 / G, sub = lane / G, l = lane - sub * G;
-  if (sub < per_warp) {
-    for (int q = (threadIdx.x >> 5) * per_warp + sub; q < ch.count; q += (blockDim.x >> 5) * per_warp) {
-      const int64_t i = (int64_t)ch.start + q;
-      const float w2 = mag(coef[off2 + (int64_t)l * M + i]) * sc;
-      const int l0 = kf[i] - org[0], l1 = kf[M + i] - org[1], ll = kf[2 * M + i] - org[2] + l;
-      float m0[JF > 0 ? JF : 1], m1[JF > 0 ? JF : 1];
+  const int step = (blockDim.x >> 5) * per_warp;
+  float* s0 = reinterpret_cast<float*>(wacc + ncell) + (threadIdx.x >> 5) * (J0 + J1) * per_warp;   // JF = 0
+  float* s1 = s0 + J0 * per_warp;
+  for (int qb = (threadIdx.x >> 5) * per_warp; qb < ch.count; qb += step) {   // warp-uniform
+    const int q = qb + sub;
+    const bool act = sub < per_warp && q < ch.count;
+    const int64_t i = (int64_t)ch.start + q;
+    float m0[JF > 0 ? JF : 1], m1[JF > 0 ? JF : kMaxJ];
+    if (JF == 0) __syncwarp();   // the strip's readers of the previous round are done
+    if (act) {
+      if (JF > 0) {
 #pragma unroll
-      for (int j = 0; j < JF; ++j) {
-        m0[j] = mag(coef[(int64_t)j * M + i]);
-        m1[j] = mag(coef[off1 + (int64_t)j * M + i]);
-      }
-#pragma unroll
-      for (int j0 = 0; j0 < (JF > 0 ? JF : kMaxJ); ++j0) {
-        if (JF == 0 && j0 >= J0) break;
-        const float w0 = (JF > 0 ? m0[j0] : mag(coef[(int64_t)j0 * M + i])) * w2;
-        uint32_t* row = wacc + ((l0 + j0) * g.P[1] + l1) * g.P[2] + ll;
-#pragma unroll
-        for (int j1 = 0; j1 < (JF > 0 ? JF : kMaxJ); ++j1) {
-          if (JF == 0 && j1 >= J1) break;
-          const float w = __fmaf_ru(JF > 0 ? m1[j1] : mag(coef[off1 + (int64_t)j1 * M + i]), w0, 8388608.0f);
-          atomicAdd(row + j1 * g.P[2], __float_as_uint(w) & 0x7fffffu);
+        for (int j = 0; j < JF; ++j) {
+          m0[j] = mag(coef[(int64_t)j * M + i]);
+          m1[j] = mag(coef[off1 + (int64_t)j * M + i]);
         }
+      } else {
+        for (int j = l; j < J0; j += G) s0[j * per_warp + sub] = mag(coef[(int64_t)j * M + i]);
+        for (int j = l; j < J1; j += G) s1[j * per_warp + sub] = mag(coef[off1 + (int64_t)j * M + i]);
+      }
+    }
+    if (JF == 0) __syncwarp();
+    if (!act) continue;
+    if (JF == 0) {
+#pragma unroll
+      for (int j = 0; j < kMaxJ; ++j) m1[j] = j < J1 ? s1[j * per_warp + sub] : 0.f;
+    }
+    const float w2 = mag(coef[off2 + (int64_t)l * M + i]) * sc;
+    const int l0 = kf[i] - org[0], l1 = kf[M + i] - org[1], ll = kf[2 * M + i] - org[2] + l;
+#pragma unroll(JF > 0 ? JF : 1)
+    for (int j0 = 0; j0 < J0; ++j0) {
+      const float w0 = (JF > 0 ? m0[j0] : s0[j0 * per_warp + sub]) * w2;
+      uint32_t* row = wacc + ((l0 + j0) * g.P[1] + l1) * g.P[2] + ll;
+#pragma unroll
+      for (int j1 = 0; j1 < (JF > 0 ? JF : kMaxJ); ++j1) {
+        if (JF == 0 && j1 >= J1) break;
+        const float w = __fmaf_ru(m1[j1], w0, 8388608.0f);
+        atomicAdd(row + j1 * g.P[2], __float_as_uint(w) & 0x7fffffu);
       }
     }
   }
@@ -957,16 +980,16 @@ int build_points(nufft_plan_t* p, const float* om, HostLists& lists) {
         p->coef, M, d, g.J[0], d > 1 ? g.J[1] : 0, d > 2 ? g.J[2] : 0, p->cmax);
     NUFFT_CUDA_TRY(p, cudaGetLastError());
     if (d == 3 && nch > 0) {
-      const size_t smem = (size_t)g.padded_cells * sizeof(uint32_t);
-      const bool eq = g.J[0] == g.J[1] && g.J[1] == g.J[2];
+      const bool fixed = g.J[0] == g.J[1] && g.J[1] == g.J[2] && g.J[0] >= 4 && g.J[0] <= 7;
+      const size_t smem = wmax_smem(g, fixed);
       auto kern = k_chunk_wmax<0>;
-      if (eq && g.J[0] == 4) kern = k_chunk_wmax<4>;
-      if (eq && g.J[0] == 5) kern = k_chunk_wmax<5>;
-      if (eq && g.J[0] == 6) kern = k_chunk_wmax<6>;
-      if (eq && g.J[0] == 7) kern = k_chunk_wmax<7>;
+      if (fixed && g.J[0] == 4) kern = k_chunk_wmax<4>;
+      if (fixed && g.J[0] == 5) kern = k_chunk_wmax<5>;
+      if (fixed && g.J[0] == 6) kern = k_chunk_wmax<6>;
+      if (fixed && g.J[0] == 7) kern = k_chunk_wmax<7>;
       NUFFT_CUDA_TRY(p, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      kern<<<(unsigned)nch, 512, smem, st>>>(p->chunks, p->kf, p->coef, p->coef_off[1], p->coef_off[2], M, g,
-                                                     p->cmax);
+      kern<<<(unsigned)nch, kWmaxThreads, smem, st>>>(p->chunks, p->kf, p->coef, p->coef_off[1], p->coef_off[2], M, g,
+                                                      p->cmax);
       NUFFT_CUDA_TRY(p, cudaGetLastError());
     }
     if (p->dcoef) {

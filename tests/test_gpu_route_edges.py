@@ -173,3 +173,32 @@ def test_3d_interpolation_routes(nf, J, M, staged):
     assert rel(got[picks], oracle.interp_V(p, z)) < TOL_V
     if "k_interp" in names:
         assert ("k_interp_chunk3d" in names) == staged, names
+
+
+# every J of the two-word bound by magnitudes in a strip of shared memory, samples aligned in
+# phase at the most loaded cell, chunks of the largest size inside one tile of 16
+@pytest.mark.parametrize("Jd,M", [((6, 5, 4), 2048), ((2, 7, 5), 1500), ((8, 8, 8), 700), ((1, 3, 1), 900),
+                                  ((6, 6, 6), 2048), ((6, 6, 6), 2049), ((4, 4, 4), 2048), ((7, 7, 7), 2048)])
+def test_3d_gridding_bound_in_one_tile(nf, Jd, M):
+    K, N = 32, 16
+    rng = np.random.default_rng(M)
+    u = np.stack([_first(J) + rng.uniform(0.1, 15.9, M) for J in Jd], 1)
+    om = (2 * np.pi / K * (u - K * (u > K / 2))).astype(np.float32)
+    p = oracle.make_plan(om, (N,) * 3, (K,) * 3, Jd)
+    first = (p.k0 + 1) % K
+    assert first.max() < 16    # one tile
+    load = np.zeros((K,) * 3)
+    for js in np.ndindex(*Jd):
+        idx = tuple((p.k0[:, a] + 1 + js[a]) % K for a in range(3))
+        np.add.at(load, idx, np.abs(np.prod([p.coef[a][:, js[a]] for a in range(3)], axis=0)))
+    cell = np.unravel_index(np.argmax(load), load.shape)
+    w = np.ones(M, dtype=np.complex128)
+    for a in range(3):
+        j = (cell[a] - (p.k0[:, a] + 1)) % K
+        w *= np.where(j < Jd[a], p.coef[a][np.arange(M), np.minimum(j, Jd[a] - 1)], 0)
+    y = np.where(np.abs(w) > 0, w / np.maximum(np.abs(w), 1e-300), 1.0).astype(np.complex64)
+    ref = oracle.gridding_VH(p, y)
+    with nf.NufftPlan(dev(om), (N,) * 3, (K,) * 3, Jd) as plan:
+        assert plan.info()["nchunks"] == (M + 2047) // 2048
+        got = plan.gridding(dev(y)).cpu().numpy()
+    assert rel(got, ref) < TOL_V
