@@ -1347,9 +1347,9 @@ k_gridding_chunk_staged(const float2* __restrict__ y_b, float2* __restrict__ til
 // warps.  A batch has CTAs enough, and the chunks of a dynamic series' frames are
 // small (30 points), so what counts is the instructions spent per CTA: eight
 // warps with staged point data (k_gridding_chunk_staged) spend most of theirs on
-// set-up, barriers and idle warps.  A single transform keeps that kernel: its
-// few CTAs are bound by latency, which staging everything at once hides better
-// (a 512^2 grid with 206,336 points: 56 us for the pair, 67 us with these).
+// set-up, barriers and idle warps.  With fewer CTAs or longer chunks latency is what
+// bounds them, and staging everything at once hides it better (one transform on a
+// 512^2 grid with 206,336 points: 56 us for the pair, 67 us with these).
 // The lane
 // layout is that of k_interp (a group of J_1 lanes per point, lane l its l-th
 // neighbour along the contiguous axis); every warp loads the next round's point
@@ -1358,8 +1358,9 @@ k_gridding_chunk_staged(const float2* __restrict__ y_b, float2* __restrict__ til
 // passes c_0[l] to the point's other lanes through a per-warp strip of shared
 // memory.  JF > 0: J_0 = J_1 = JF; JF = 0: any J, c_0 is loaded in the round.
 constexpr int kBatchWarps2d = 2;
-// Batches take k_gridding_chunk2d below this mean chunk and above this many CTAs.
-// Measured, k_gridding_chunk2d against k_gridding_chunk_staged: 30 points per
+// k_gridding_chunk2d runs below this mean chunk and above this many CTAs, batches and
+// single transforms alike (one of 300,000 points on 1000^2, 30 per chunk, 31.9 us
+// against 41.6 staged).  Measured, k_gridding_chunk2d against k_gridding_chunk_staged: 30 points per
 // chunk, 32 coils 76 us against 95; 108 points, 16 images 55 against 46; 105
 // points, 8 coils (1968 CTAs) 20 against 14.
 constexpr int64_t kBatchMaxMean = 64;
@@ -1843,7 +1844,7 @@ cudaError_t launch_chunks(const nufft_plan_t* p, const float2* y, float2* tiles,
   const bool j6 = all_j_equal(p->g, 6);
   cudaError_t e;
   if constexpr (D == 2 && !FUSED) {
-    // few points per chunk and CTAs enough: two warps per CTA
+    // few points per chunk and CTAs enough, batch or not: two warps per CTA
     if (p->nchunks * nb >= kBatchMinCtas && p->M <= kBatchMaxMean * p->nchunks) {
       auto go = [&](auto kern, int nstrip) {
         const size_t smem = (size_t)p->g.padded_cells * Fix<2>::kWords * sizeof(int) +

@@ -83,6 +83,18 @@ def test_2d_many_neighbours(nf, Jd, Kd):
         assert rel(plan.gridding(dev(y)).cpu().numpy(), oracle.gridding_VH(p, y)) < TOL_V
 
 
+# one transform whose small chunks go to the two-warp gridding kernel
+def test_2d_single_transform_of_small_chunks(nf):
+    Kd, Nd, M = (1000, 972), (500, 486), 250001
+    om = W.uniform_random_om(M, 2, seed=8)
+    p = oracle.make_plan(om, Nd, Kd, (4, 4))
+    y = cn(M, 7)
+    with nf.NufftPlan(dev(om), Nd, Kd, (4, 4)) as plan:
+        nch = plan.info()["nchunks"]
+        assert nch >= 32 * 152 and M <= 64 * nch   # the rule for that kernel
+        assert rel(plan.gridding(dev(y)).cpu().numpy(), oracle.gridding_VH(p, y)) < TOL_V
+
+
 # 1D: one tile's list of 1 to 40 chunks over four thread groups, three pairs in flight.  A
 # chunk's sums round by up to 2^-31 B per contribution, B < 2 max|c| sum(|Re y| + |Im y|) over its
 # points; a wrong list is off by whole contributions.
@@ -202,3 +214,15 @@ def test_3d_gridding_bound_in_one_tile(nf, Jd, M):
         assert plan.info()["nchunks"] == (M + 2047) // 2048
         got = plan.gridding(dev(y)).cpu().numpy()
     assert rel(got, ref) < TOL_V
+
+
+# the stable sort by tile around the size at which its tile changes
+@pytest.mark.parametrize("M", [(1 << 18) - 1, 1 << 18, (1 << 18) + 1, 5])
+def test_sort_by_tile(nf, M):
+    om = W.uniform_random_om(M, 2, seed=12)
+    with nf.NufftPlan(dev(om), (64, 64), (128, 128), (6, 6)) as plan:
+        kf, _, _, perm = plan.interpolator()
+    k = kf.numpy()[perm.numpy()] // 16
+    tile = k[:, 0] * 8 + k[:, 1]
+    assert (np.diff(tile) >= 0).all()
+    np.testing.assert_array_equal(np.sort(perm.numpy()), np.arange(M))
