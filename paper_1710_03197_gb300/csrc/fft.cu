@@ -23,7 +23,7 @@
 // are; the hand-offs between stages go through two shared-memory buffers used
 // in turn (one buffer where there is one hand-off), one barrier per hand-off.
 // Twiddles are computed in registers.
-// Other line lengths (even, prime factors 2, 3 and 5) run stages of radices 2 to 16
+// Other line lengths (even, prime factors 2, 3 and 5) run stages of radices 2 to 8
 // (k_fft_mixed).
 #include <type_traits>
 

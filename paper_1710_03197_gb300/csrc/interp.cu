@@ -284,7 +284,7 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
   return r;
 }
 
-// 3D with every J = JF (4 to 7): as k_interp_chunk, and every warp keeps the next
+// 3D with every J = JF (4 to 7): as k_interp_chunk3d_any, and every warp keeps the next
 // round's point data in flight while it gathers this one's, with no barrier
 // between rounds: lane l of a point loads the l-th coefficient of each axis into
 // registers a round ahead; the axis-0 and axis-1 ones reach the point's other
@@ -752,7 +752,7 @@ __device__ __forceinline__ float2 fix_value(const int* acc, int ncell, int c, co
 // The accumulator words are held as planes (word k of every cell, then word
 // k + 1, ...) so that the J_last lanes of a point hit J_last consecutive banks
 // per atomic.
-template <int D, int JF>
+template <int D>
 struct GridChunkCfg {
   static constexpr int kThreads = D == 3 ? 512 : 256;
   static constexpr int kMinBlocks = D == 3 ? 2 : 4;
@@ -798,7 +798,7 @@ __device__ __forceinline__ void scatter_chunk(int* acc, const int ncell, const f
     const int ll = P.kf[(int64_t)(D - 1) * P.M + i] - org[D - 1] + l;
     const float2 cl = P.coef[P.coef_off[D - 1] + (int64_t)l * P.M + i];
     const float2 yl = cmulc(cl, yv);  // conj(c_last) * y
-    if (D == 1) {
+    if constexpr (D == 1) {
       fix_add<WORDS>(acc, ncell, ll, yl);
     } else {
       const int l0 = P.kf[i] - org[0];
@@ -827,15 +827,6 @@ __device__ __forceinline__ void scatter_chunk(int* acc, const int ncell, const f
   }
 }
 
-// 3D chunk pass with every J = JF (4 to 7): as k_gridding_chunk, but a chunk
-// that sums in two words keeps its samples in shared memory (they are gathered
-// once, for the scale; the third word's space holds them), and every warp keeps
-// the next round's coefficients in flight while it scatters this one's: lane l
-// of a point loads the l-th coefficient of each axis into registers a round
-// ahead, and the axis-0 and axis-1 ones are passed to the point's other lanes
-// through a per-warp strip of shared memory.  A chunk that needs three words
-// takes scatter_chunk.  128^3 kooshball: 517 us with three words throughout, 324 us
-// so, with the shared-memory pipe 78 % and the issue slots 66 % busy.
 // rn(x) as an integer for |x| < 1.2e9 on the FP32 and integer pipes: three
 // additions and a shift-add, against one F2I, which the conversion unit issues
 // at one warp per two cycles and SM.  t holds x rounded to a multiple of 512
@@ -850,6 +841,15 @@ __device__ __forceinline__ int round_int(float x) {
   return (__float_as_int(t) << 9) + __float_as_int(l);
 }
 
+// 3D chunk pass with every J = JF (4 to 7): as k_gridding_chunk, but a chunk
+// that sums in two words keeps its samples in shared memory (they are gathered
+// once, for the scale; the third word's space holds them), and every warp keeps
+// the next round's coefficients in flight while it scatters this one's: lane l
+// of a point loads the l-th coefficient of each axis into registers a round
+// ahead, and the axis-0 and axis-1 ones are passed to the point's other lanes
+// through a per-warp strip of shared memory.  A chunk that needs three words
+// takes scatter_chunk.  128^3 kooshball: 517 us with three words throughout, 324 us
+// so, with the shared-memory pipe 78 % and the issue slots 66 % busy.
 template <int JF, int TF>
 __device__ __forceinline__ void scatter_chunk3d(int* acc, const int ncell, const float2* s_y, float2* strip,
                                                 const Chunk& ch, const Points& P, const Geom& g,
@@ -964,18 +964,16 @@ k_gridding_chunk3d(const float2* __restrict__ y_b, float2* __restrict__ tiles_b,
 
 // 1D chunk pass, and the 3D one for the J that k_gridding_chunk3d does not take
 // (2D: k_gridding_chunk_staged).
-template <int D, int JF, int TF>
-__global__ void __launch_bounds__(GridChunkCfg<D, JF>::kThreads, GridChunkCfg<D, JF>::kMinBlocks)
+template <int D, int JF>
+__global__ void __launch_bounds__(GridChunkCfg<D>::kThreads, GridChunkCfg<D>::kMinBlocks)
 k_gridding_chunk(const float2* __restrict__ y_b, float2* __restrict__ tiles_b, const Chunk* __restrict__ chunks,
                  const Points P, const Geom g, int64_t ybs, int64_t tbs) {
   static_assert(D != 2, "2D has its own kernel");
-  static_assert(TF == 0 || JF > 0, "a fixed tile needs a fixed J");
-  constexpr int PF = TF > 0 ? TF + JF - 1 : 0;   // padded edge when fixed
   extern __shared__ int acc[];
   __shared__ float red[32];
   const float2* __restrict__ y = y_b + (int64_t)blockIdx.y * ybs;
   float2* __restrict__ tiles = tiles_b + (int64_t)blockIdx.y * tbs;
-  const int ncell = TF > 0 ? (D == 1 ? PF : PF * PF * PF) : (int)g.padded_cells;
+  const int ncell = (int)g.padded_cells;
   const Chunk ch = chunks[blockIdx.x];
   for (int c = threadIdx.x; c < Fix<D>::kWords * ncell; c += blockDim.x) acc[c] = 0;
 
@@ -1001,8 +999,8 @@ k_gridding_chunk(const float2* __restrict__ y_b, float2* __restrict__ tiles_b, c
     }
   }
   if (cs.finite) {   // CTA-uniform
-    if (D < 3 || cs.two) scatter_chunk<D, JF, TF, 2>(acc, ncell, y, ch, P, g, org, cs.S);
-    else scatter_chunk<D, JF, TF, 3>(acc, ncell, y, ch, P, g, org, cs.S);
+    if (D < 3 || cs.two) scatter_chunk<D, JF, 0, 2>(acc, ncell, y, ch, P, g, org, cs.S);
+    else scatter_chunk<D, JF, 0, 3>(acc, ncell, y, ch, P, g, org, cs.S);
   }
   __syncthreads();
   float2* out = tiles + (int64_t)ch.slot * g.padded_cells;
@@ -1010,6 +1008,7 @@ k_gridding_chunk(const float2* __restrict__ y_b, float2* __restrict__ tiles_b, c
 }
 
 // ---------------------------------------------------------------- gridding, tile reduction
+// 1D and 2D (3D: k_gridding_reduce3d; 2D batches: k_gridding_reduce2d).
 // One CTA per tile: grid cell c of tile b is the sum over e in {0,1}^d of the
 // padded tiles of bin b - e (wrapped per dimension) at local position
 // c - origin(b) + e * T, when that position lies inside the padded tile.  Each
@@ -1039,24 +1038,15 @@ template <int D, int CPT, int TF>
 __device__ __forceinline__ void reduce_cells(const Geom& g, const int (&bc)[kMaxDim], int tg, int gsize,
                                              int tile_cells, int cend, int (&loc0)[CPT], unsigned (&emask)[CPT],
                                              int (&goff)[CPT]) {
-  const int P1 = D > 1 ? g.P[1] : 1, P2 = D > 2 ? g.P[2] : 1;
+  static_assert(D < 3, "3D has its own kernel");
+  const int P1 = D > 1 ? g.P[1] : 1;
   // TF > 0: every tile edge is TF, so the cell decompositions below divide by constants
-  const int T1 = D > 1 ? (TF > 0 ? TF : g.T[1]) : 1, T2 = D > 2 ? (TF > 0 ? TF : g.T[2]) : 1;
+  const int T1 = D > 1 ? (TF > 0 ? TF : g.T[1]) : 1;
 #pragma unroll
   for (int k = 0; k < CPT; ++k) {
     const int c = min(tg + k * gsize, tile_cells - 1);
-    int lc[3] = {0, 0, 0};
-    if (D == 1) {
-      lc[0] = c;
-    } else if (D == 2) {
-      lc[1] = c % T1;
-      lc[0] = c / T1;
-    } else {
-      lc[2] = c % T2;
-      lc[1] = (c / T2) % T1;
-      lc[0] = c / (T2 * T1);
-    }
-    loc0[k] = D == 1 ? lc[0] : (D == 2 ? lc[0] * P1 + lc[1] : (lc[0] * P1 + lc[1]) * P2 + lc[2]);
+    const int lc[2] = {c / T1, c % T1};   // 1D: T1 = 1
+    loc0[k] = lc[0] * P1 + lc[1];
     // neighbour e reaches the cell iff every axis a with e_a = 1 has the cell
     // within J - 1 of the tile's low edge; with those axes as the bits of
     // `near` (e's bit order), the mask is the set of subsets of near
@@ -1088,14 +1078,13 @@ __device__ __forceinline__ void reduce_tile(const float2* __restrict__ tiles, co
       rem /= g.nb[a];
     }
   }
-  const int P1 = D > 1 ? g.P[1] : 1, P2 = D > 2 ? g.P[2] : 1;
   if (threadIdx.x < (1 << D)) {
     const int e = threadIdx.x;
     int src = 0, delta = 0;
     for (int a = 0; a < D; ++a) {
       const int ea = (e >> (D - 1 - a)) & 1;
       src = src * g.nb[a] + (bc[a] - ea + g.nb[a]) % g.nb[a];
-      const int pstride = a == D - 1 ? 1 : (a == D - 2 ? g.P[D - 1] : P1 * P2);
+      const int pstride = a == D - 1 ? 1 : g.P[D - 1];
       delta += ea * g.T[a] * pstride;
     }
     s_q0[e] = bin_chunk[src];
@@ -1696,7 +1685,6 @@ cudaError_t interp_chunks(const nufft_plan_t* p, const float2* grid, float2* y, 
   if (p->nchunks == 0) return cudaSuccess;
   const Points P = points_view(p);
   const dim3 gd((unsigned)p->nchunks, (unsigned)nb);
-  const bool j6 = all_j_equal(p->g, 6);
   bool t16 = true;
   for (int a = 0; a < D; ++a) t16 = t16 && p->g.T[a] == 16;
   if constexpr (D == 2) {
@@ -1841,7 +1829,6 @@ cudaError_t launch_chunks(const nufft_plan_t* p, const float2* y, float2* tiles,
   if (p->nchunks == 0) return cudaSuccess;
   const Points P = points_view(p);
   const dim3 gd((unsigned)p->nchunks, (unsigned)nb);
-  const bool j6 = all_j_equal(p->g, 6);
   cudaError_t e;
   if constexpr (D == 2 && !FUSED) {
     // few points per chunk and CTAs enough, batch or not: two warps per CTA
@@ -1888,15 +1875,17 @@ cudaError_t launch_chunks(const nufft_plan_t* p, const float2* y, float2* tiles,
   } else {
     static_assert(!FUSED, "the fused V^H V pass is 2D only");
     const size_t smem = (size_t)p->g.padded_cells * Fix<D>::kWords * sizeof(int);
-    constexpr int NT = GridChunkCfg<D, 6>::kThreads;
+    const int J = all_j_equal(p->g, p->g.J[0]) ? p->g.J[0] : 0;
     if constexpr (D == 3) {
-      const int J = all_j_equal(p->g, p->g.J[0]) ? p->g.J[0] : 0;
       if (J >= 4 && J <= 7) return launch_chunks3d(p, y, tiles, gd, J, ybs, tbs);
     }
-    auto kern = D == 1 && j6 ? k_gridding_chunk<D, (D == 1 ? 6 : 0), 0> : k_gridding_chunk<D, 0, 0>;
+    auto kern = k_gridding_chunk<D, 0>;
+    if constexpr (D == 1) {
+      if (J == 6) kern = k_gridding_chunk<D, 6>;
+    }
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<gd, NT, smem, p->stream>>>(y, tiles, p->chunks, P, p->g, ybs, tbs);
+    kern<<<gd, GridChunkCfg<D>::kThreads, smem, p->stream>>>(y, tiles, p->chunks, P, p->g, ybs, tbs);
   }
   return cudaGetLastError();
 }
