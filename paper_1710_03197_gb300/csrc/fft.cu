@@ -498,7 +498,7 @@ cudaError_t launch_LE(const FftArgs& A, int nb, cudaStream_t st, int64_t* nblock
   if constexpr (!STRIDED) {
     if (A.pro_p || A.epi_part) return go(k_fft_pass<L, E, STRIDED, INV, true, 0>);
   } else {
-    constexpr int kFull = E == 16 ? 4 : 3;
+    constexpr int kFull = E == 16 && L < 512 ? 4 : 3;
     if (wlog == kFull) return go(k_fft_pass<L, E, STRIDED, INV, false, kFull>);
   }
   return go(k_fft_pass<L, E, STRIDED, INV, false, 0>);
@@ -508,15 +508,17 @@ cudaError_t launch_LE(const FftArgs& A, int nb, cudaStream_t st, int64_t* nblock
 // the GPU: one hand-off instead of two, fewer twiddles per value, and 128-byte rows
 // (with the hand-offs above, a 256^3 grid's transform 105 -> 81 us forward, 104 ->
 // 69 us inverse, L2 flushed; the error against 64 bits falls by a fifth).  Lines of
-// 512 points need two hand-offs either way: 2 % faster with sixteen values on 32
-// coils of 512^2, but a smooth image's samples are 1.22 times further off.  The
-// contiguous passes lose more to the registers and the scaling's loads, and a small
-// pass is bound by latency: all these take eight, with twice the warps.
+// 512 points need two hand-offs either way and take 64-byte rows: 32 coils of 512^2
+// 28.0 -> 26.6 us forward, 26.0 -> 24.3 inverse, but a smooth image's samples are
+// 1.22 times further off, so the inverse passes alone have them (their error is that
+// of eight values).  The contiguous passes lose more to the registers and the
+// scaling's loads, and a small pass is bound by latency: all these take eight, with
+// twice the warps.
 constexpr int64_t kWideWarps = 8 * 152;
 
 template <int L, bool STRIDED, bool INV>
 cudaError_t launch_L(const FftArgs& A, int nb, cudaStream_t st, int64_t* nblocks, bool query) {
-  if constexpr (STRIDED && (L == 128 || L == 256)) {
+  if constexpr (STRIDED && (L == 128 || L == 256 || (L == 512 && INV))) {
     if (A.nouter * A.inner * nb * (L / 16) >= kWideWarps * 32 && A.inner % 16 == 0)
       return launch_LE<L, 16, STRIDED, INV>(A, nb, st, nblocks, query);
   }
